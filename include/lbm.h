@@ -165,6 +165,9 @@ int lbm_set_storage(lbm_handle h, int storage);
 /* Enqueue all later device work on this cudaStream_t (not owned; NULL = the
  * legacy default stream, which also disables CUDA-graph replay). */
 int lbm_set_stream(lbm_handle h, void* stream);
+/* The stream the handle's work goes to, for ordering a caller's own work
+ * around it. */
+int lbm_get_stream(lbm_handle h, void** stream);
 
 /* Bytes of the population store: (Q_f + Q_g) * nx*ny*nz * element size. */
 int lbm_required_bytes(lbm_handle h, size_t* bytes);

@@ -15,6 +15,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_dispatch.h"
+#include "lbm_halo.cuh"
 #include "lbm_kernels.cuh"
 #include "lbm_stage.cuh"
 
@@ -91,6 +92,7 @@ struct lbm_ctx {
     int pairing = LBM_PAIRING_ALL;   // two nodes per thread (16-bit storage, even nx)
     bool tile_staging = false;        // bulk-copy staged kernel where it applies
     bool slab = false;                // z-slab: planes 0 and nz - 1 are ghost planes (lbm_set_slab)
+    bool stage_used = false;          // the staged kernel, the one that can raise d_err, has been launched
     int stage_grid = 0;               // persistent grid of the staged kernel (0: not derived yet)
     int* d_err = nullptr;             // device flag raised by a bounded wait that ran out
     uint32_t stage_spin = 1u << 22;   // mbarrier polls per wait
@@ -391,6 +393,7 @@ cudaError_t launch_staged(lbm_ctx* h, int odd, int W, cudaStream_t s)
         const size_t cap = (size_t)(h->num_sms > 0 ? h->num_sms : 1) * (size_t)occ;
         h->stage_grid = (int)(a.ntiles < cap ? a.ntiles : cap);
     }
+    h->stage_used = true;
     void* args[] = {&a};
     return cudaLaunchKernel(k, dim3((unsigned)h->stage_grid), dim3((unsigned)stage_threads(W)), args, smem, s);
 }
@@ -494,25 +497,56 @@ int check_device_buffer(const lbm_ctx* h, const void* p)
     return LBM_OK;
 }
 
-// Halo buffer <-> plane z of the store: the f slots with e_z = sign, then the
-// g slots with e_z = sign, nx*ny elements each (one contiguous run per slot
-// and plane in the store). pack = store -> buffer.
-int halo_copy(lbm_ctx* h, int z, int sign, void* buf, bool pack)
+// One side of a halo copy: plane z of the store's f slots with e_z = sign, then
+// of its g slots with e_z = sign, nx*ny elements each (one contiguous run per
+// slot and plane in the store). Returns the number of runs.
+int halo_side(lbm_ctx* h, int z, int sign, const void* buf, HaloSide* out)
 {
     const size_t es = elem_size(h->p.storage);
     const size_t plane = (size_t)h->p.nx * (size_t)h->p.ny * es;
     int slots[27];
-    char* b = static_cast<char*>(buf);
+    int runs = 0;
     for (int part = 0; part < 2; ++part) {
         const int q = part ? h->q.qg : h->q.qf;
         char* base = static_cast<char*>(part ? g_ptr(h) : f_ptr(h));
         const int n = halo_slots(q, sign, slots);
-        for (int k = 0; k < n; ++k) {
-            char* at = base + ((size_t)slots[k] * h->geo.n3) * es + (size_t)z * plane;
-            LBM_CUDA(cudaMemcpyAsync(pack ? b : at, pack ? at : b, plane, cudaMemcpyDeviceToDevice, h->stream),
-                     "halo copy");
-            b += plane;
-        }
+        for (int k = 0; k < n; ++k) out->run[runs++] = base + ((size_t)slots[k] * h->geo.n3) * es + (size_t)z * plane;
+    }
+    out->buffer = static_cast<char*>(const_cast<void*>(buf));
+    return runs;
+}
+
+// Both halo buffers of a slab in one launch: `lower` holds the slots of sign
+// `sl` at plane zl, `upper` those of sign su at zu. Buffers of a pack that
+// overlap take one launch each, in order, so that the upper one's bytes stand.
+int halo_copy(lbm_ctx* h, int zl, int sl, const void* lower, int zu, int su, const void* upper, bool pack)
+{
+    HaloArgs a{};
+    a.plane = (size_t)h->p.nx * (size_t)h->p.ny * elem_size(h->p.storage);
+    a.pack = pack ? 1 : 0;
+    const int runs = halo_side(h, zl, sl, lower, &a.side[0]);
+    halo_side(h, zu, su, upper, &a.side[1]);
+    // the widest type that every address is a multiple of: the runs lie at
+    // whole planes from the store's start (and the g part at whole elements)
+    uintptr_t bits = (uintptr_t)a.plane;
+    for (const HaloSide& s : a.side) {
+        bits |= (uintptr_t)s.buffer;
+        for (int k = 0; k < runs; ++k) bits |= (uintptr_t)s.run[k];
+    }
+    const int width = bits % 16 == 0 ? 16 : bits % 4 == 0 ? 4 : bits % 2 == 0 ? 2 : 1;
+    const size_t n = a.plane / (size_t)width;
+    const size_t want = (n + 4 * kHaloThreads - 1) / (4 * kHaloThreads);
+    const unsigned bx = (unsigned)(want < 1024 ? want : 1024);
+    const char* b0 = a.side[0].buffer;
+    const char* b1 = a.side[1].buffer;
+    const size_t bytes = (size_t)runs * a.plane;
+    const bool overlap = pack && b0 < b1 + bytes && b1 < b0 + bytes;
+    for (int launch = 0; launch < (overlap ? 2 : 1); ++launch) {
+        if (launch) a.side[0] = a.side[1];
+        void* args[] = {&a};
+        LBM_CUDA(cudaLaunchKernel(halo_kernel(width), dim3(bx, (unsigned)runs, overlap ? 1u : 2u), dim3(kHaloThreads),
+                                  args, 0, h->stream),
+                 "halo copy");
     }
     return LBM_OK;
 }
@@ -664,6 +698,13 @@ int lbm_set_stream(lbm_handle h, void* stream)
     }
     h->stream = static_cast<cudaStream_t>(stream);
     h->own_stream = false;
+    return LBM_OK;
+}
+
+int lbm_get_stream(lbm_handle h, void** stream)
+{
+    if (!h || !stream) return fail(LBM_EINVAL, "null argument");
+    *stream = h->stream;
     return LBM_OK;
 }
 
@@ -886,6 +927,8 @@ int lbm_synchronize(lbm_handle h)
     if (rc) return rc;
     LBM_CUDA(cudaStreamSynchronize(h->stream), "stream synchronize");
     if (h->copy_stream) LBM_CUDA(cudaStreamSynchronize(h->copy_stream), "copy stream synchronize");
+    // only the staged kernel raises the flag: other handles are spared its copy
+    if (!h->stage_used) return LBM_OK;
     int err = 0;
     LBM_CUDA(cudaMemcpy(&err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost), "error flag read");
     if (err) {
@@ -1285,8 +1328,8 @@ int lbm_halo_pack(lbm_handle h, int phase, void* to_lower, void* to_upper)
     const int top = h->p.nz - 1;
     // phase 0: own boundary planes (plane 1: e_z = +1 slots; plane nz-2: e_z = -1)
     // phase 1: ghost planes (plane 0: e_z = -1 slots; plane nz-1: e_z = +1)
-    if ((rc = halo_copy(h, phase ? 0 : 1, phase ? -1 : +1, to_lower, true))) return rc;
-    return halo_copy(h, phase ? top : top - 1, phase ? +1 : -1, to_upper, true);
+    return halo_copy(h, phase ? 0 : 1, phase ? -1 : +1, to_lower, phase ? top : top - 1, phase ? +1 : -1, to_upper,
+                     true);
 }
 
 int lbm_halo_unpack(lbm_handle h, int phase, const void* from_lower, const void* from_upper)
@@ -1301,8 +1344,8 @@ int lbm_halo_unpack(lbm_handle h, int phase, const void* from_lower, const void*
     const int top = h->p.nz - 1;
     // phase 0: into the ghost planes (plane 0: e_z = -1 slots; plane nz-1: e_z = +1)
     // phase 1: into the own boundary planes (plane 1: e_z = +1; plane nz-2: e_z = -1)
-    if ((rc = halo_copy(h, phase ? 1 : 0, phase ? +1 : -1, const_cast<void*>(from_lower), false))) return rc;
-    return halo_copy(h, phase ? top - 1 : top, phase ? -1 : +1, const_cast<void*>(from_upper), false);
+    return halo_copy(h, phase ? 1 : 0, phase ? +1 : -1, from_lower, phase ? top - 1 : top, phase ? -1 : +1, from_upper,
+                     false);
 }
 
 int lbm_set_graphs(lbm_handle h, int enable)

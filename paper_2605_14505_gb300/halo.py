@@ -18,6 +18,12 @@ The schedule is the same whatever moves the buffers:
 A backend holds one slab and offers: halo_bytes, new_buffer(), pack(phase,
 to_lower, to_upper), unpack(phase, from_lower, from_upper), step() (one AA
 step), synchronize(). LibrarySlab is the backend of the CUDA library.
+
+A backend whose work runs on a stream also offers publish() (the current
+stream waits for the slab's work so far) and follow() (the slab's work from
+here on waits for the current stream). An exchange is then ordered on the
+device: publish after pack, move the buffers on the current stream, follow
+before unpack. Without them the exchange waits on the host (synchronize).
 """
 from __future__ import annotations
 
@@ -38,10 +44,27 @@ class LibrarySlab:
         self.sim = sim
         lbm.lbm_set_slab(sim.h, True)
         self.halo_bytes = lbm.lbm_halo_bytes(sim.h)
+        self._wrapped = (None, None)
         self.odd = lbm.lbm_step_count(sim.h) & 1
 
     def new_buffer(self):
-        return self._torch.empty(self.halo_bytes, dtype=self._torch.uint8, device="cuda")
+        buf = self._torch.empty(self.halo_bytes, dtype=self._torch.uint8, device="cuda")
+        self.follow()    # the memory may have served the current stream before
+        return buf
+
+    def _stream(self):
+        """The handle's stream, asked for each time: it may have been set again."""
+        ptr = self._lbm.lbm_get_stream(self.sim.h)
+        if self._wrapped[0] != ptr:
+            cuda = self._torch.cuda
+            self._wrapped = (ptr, cuda.ExternalStream(ptr) if ptr else cuda.default_stream())
+        return self._wrapped[1]
+
+    def publish(self):
+        self._torch.cuda.current_stream().wait_stream(self._stream())
+
+    def follow(self):
+        self._stream().wait_stream(self._torch.cuda.current_stream())
 
     def pack(self, phase, to_lower, to_upper):
         self._lbm.lbm_halo_pack(self.sim.h, phase, to_lower.data_ptr(), to_upper.data_ptr())
@@ -55,6 +78,18 @@ class LibrarySlab:
 
     def synchronize(self):
         self._lbm.lbm_synchronize(self.sim.h)
+
+
+def _publish(b):
+    """The work of slab b so far, done before what the current stream (or, without one, the host) does next."""
+    (getattr(b, "publish", None) or b.synchronize)()
+
+
+def _follow(b):
+    """What slab b does next, after what the current stream has been given (a host copy is done when it returns)."""
+    follow = getattr(b, "follow", None)
+    if follow is not None:
+        follow()
 
 
 def _copy(dst, src):
@@ -72,18 +107,31 @@ class LocalSlabs:
         self.b = list(backends)
         self.buf = [{k: b.new_buffer() for k in ("to_lower", "to_upper", "from_lower", "from_upper")}
                     for b in self.b]
+        # On one device a slab unpacks straight from its neighbours' outgoing
+        # buffers, a set per phase: a set is filled again only after the other
+        # phase's exchange (or a host wait), which every slab's work has
+        # passed by then. Otherwise the buffers are copied.
+        self.direct = (all(hasattr(b, "follow") for b in self.b)
+                       and len({x.device for bf in self.buf for x in bf.values()}) == 1)
 
     def _exchange(self, phase):
         n = len(self.b)
+        low, up = ("from_lower", "from_upper") if self.direct and phase else ("to_lower", "to_upper")
         for b, bf in zip(self.b, self.buf):
-            b.pack(phase, bf["to_lower"], bf["to_upper"])
+            b.pack(phase, bf[low], bf[up])
         for b in self.b:
-            b.synchronize()
-        for r in range(n):
-            _copy(self.buf[r]["from_lower"], self.buf[(r - 1) % n]["to_upper"])
-            _copy(self.buf[r]["from_upper"], self.buf[(r + 1) % n]["to_lower"])
-        for b, bf in zip(self.b, self.buf):
-            b.unpack(phase, bf["from_lower"], bf["from_upper"])
+            _publish(b)
+        if not self.direct:
+            for r in range(n):
+                _copy(self.buf[r]["from_lower"], self.buf[(r - 1) % n]["to_upper"])
+                _copy(self.buf[r]["from_upper"], self.buf[(r + 1) % n]["to_lower"])
+        for b in self.b:
+            _follow(b)
+        for r, (b, bf) in enumerate(zip(self.b, self.buf)):
+            if self.direct:
+                b.unpack(phase, self.buf[(r - 1) % n][up], self.buf[(r + 1) % n][low])
+            else:
+                b.unpack(phase, bf["from_lower"], bf["from_upper"])
 
     def step(self, nsteps: int = 1):
         for _ in range(nsteps):
@@ -123,7 +171,7 @@ class SlabExchange:
 
     def _exchange(self, phase):
         self.b.pack(phase, self.to_lower, self.to_upper)
-        self.b.synchronize()
+        _publish(self.b)
         if self.world == 1:
             _copy(self.from_lower, self.to_upper)
             _copy(self.from_upper, self.to_lower)
@@ -138,6 +186,7 @@ class SlabExchange:
                    dist.P2POp(dist.irecv, self.from_lower, lower, self.group, 1)]
             for req in dist.batch_isend_irecv(ops):
                 req.wait()
+        _follow(self.b)
         self.b.unpack(phase, self.from_lower, self.from_upper)
 
     def step(self, nsteps: int = 1):

@@ -109,6 +109,7 @@ _SIGS = {
     "lbm_get_params": ([_H, ctypes.POINTER(lbm_params)], ctypes.c_int),
     "lbm_set_storage": ([_H, ctypes.c_int], ctypes.c_int),
     "lbm_set_stream": ([_H, ctypes.c_void_p], ctypes.c_int),
+    "lbm_get_stream": ([_H, ctypes.POINTER(ctypes.c_void_p)], ctypes.c_int),
     "lbm_required_bytes": ([_H, ctypes.POINTER(ctypes.c_size_t)], ctypes.c_int),
     "lbm_attach": ([_H, ctypes.c_void_p, ctypes.c_size_t], ctypes.c_int),
     "lbm_init_tgv": ([_H, ctypes.c_uint64, ctypes.c_double], ctypes.c_int),
@@ -260,6 +261,12 @@ def lbm_set_storage(h, storage):
 
 def lbm_set_stream(h, stream_ptr: int):
     _check(load_library().lbm_set_stream(h, ctypes.c_void_p(stream_ptr)))
+
+
+def lbm_get_stream(h) -> int:
+    s = ctypes.c_void_p()
+    _check(load_library().lbm_get_stream(h, ctypes.byref(s)))
+    return s.value or 0
 
 
 def lbm_required_bytes(h) -> int:
