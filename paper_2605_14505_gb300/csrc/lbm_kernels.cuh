@@ -231,15 +231,78 @@ struct StepArgs {
     Phys ph;
     DiagSink dg;      // used by the diagnosing variants only
     int z0;           // first z-plane of the launch (1 for a z-slab with ghost planes, else 0)
+    // flat launches (flat > 0): threads number the plane's units (nodes, or
+    // pairs of nodes) row by row, flat of them in rows of flat_row;
+    // r / flat_row = umulhi(r, flat_mul) >> flat_shift for r < 2^31
+    uint32_t flat, flat_row, flat_mul, flat_shift;
+};
+
+// A thread's unit (xu, y) of its plane; false outside it. Shaped launches
+// tile the plane in blocks of blockDim.x x blockDim.y. The plain step kernels
+// know their launch at compile time (as a run-time choice it cost the 16-bit
+// pair kernel 12 bytes of spill and 0.3 % at 256^3), the diagnosing ones ask.
+enum StepLaunch : int { kShaped = 0, kFlat = 1, kAsked = 2 };
+template <int LAUNCH>
+__device__ __forceinline__ bool step_unit(const StepArgs& a, int xunits, int& xu, int& y, uint32_t tx)
+{
+    if (LAUNCH == kFlat || (LAUNCH == kAsked && a.flat)) {
+        const uint32_t r = blockIdx.x * blockDim.x + tx;
+        y = (int)(__umulhi(r, a.flat_mul) >> a.flat_shift);
+        xu = (int)(r - (uint32_t)y * a.flat_row);
+        return r < a.flat;
+    }
+    xu = (int)(blockIdx.x * blockDim.x + tx);
+    y = (int)(blockIdx.y * blockDim.y + threadIdx.y);
+    return xu < xunits && y < a.geo.ny;
+}
+
+// Programmatic dependent launch: once every block of a step has come to its
+// stores, the next step's blocks may take free SM slots; they wait there until
+// this launch is complete and its stores visible, so only the launch itself
+// overlaps. Asked for at the start of a step instead, the waiting blocks crowd
+// the few free SMs of a small lattice (D3Q27xD3Q19 32^3 5.4 against 3.3 us per
+// step; 3.5 without overlap). Without the launch attribute both are no-ops.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Where a step kernel's thread stands, worked out again for its stores from
+// the (laundered) thread index: carried through the collision instead, the two
+// coordinates cost registers that the 80-register kernels do not have (FP32
+// Guo odd step 68 bytes of spill, the 16-bit pair kernels 4 to 48).
+template <int LAUNCH>
+struct StepPlace {
+    const StepArgs& a;
+    int per;   // nodes per unit
+    __device__ __forceinline__ void operator()(int& x, int& y, int& z) const
+    {
+        launch_dependents();
+        if constexpr (LAUNCH == kShaped) {
+            x = (int)launder(x);
+            y = (int)launder(y);
+        } else {
+            step_unit<LAUNCH>(a, 0, x, y, launder(threadIdx.x));
+            x *= per;
+            y = (int)launder(y);
+        }
+        z = (int)launder(z);
+    }
+};
+struct SamePlace {
+    __device__ __forceinline__ void operator()(int& x, int& y, int& z) const
+    {
+        x = (int)launder(x);
+        y = (int)launder(y);
+        z = (int)launder(z);
+    }
 };
 
 // The fused AA update of one node: load the QF + QG populations (coalesced
 // along x), moments, coupled rho'/u solve, f and g collisions, store.
 // hook(h, m) runs between the moments and the collisions (the diagnosing
 // step kernels read the pre-collision state there).
-template <class P, int FORCING, class T, bool ODD, class Hook>
+template <class P, int FORCING, class T, bool ODD, class Hook, class Place = SamePlace>
 __device__ __forceinline__ void update_node(void* fv, void* gv, const Geometry& geo, const Phys& ph, int x,
-                                            int y, int z, Hook&& hook)
+                                            int y, int z, Hook&& hook, Place place = Place())
 {
     const NodeAddr a = node_addr<T>(geo, x, y, z);
     T* __restrict__ f = static_cast<T*>(fv);
@@ -250,7 +313,8 @@ __device__ __forceinline__ void update_node(void* fv, void* gv, const Geometry& 
     load_node<typename P::LF, ODD, T>(f, n3, a, h);
     load_node<typename P::LG, ODD, T>(g, n3, a, k);
     collide_node<P, FORCING, kExact>(h, k, ph, hook);
-    const NodeAddr b = node_addr<T>(geo, (int)launder(x), (int)launder(y), (int)launder(z));
+    place(x, y, z);
+    const NodeAddr b = node_addr<T>(geo, x, y, z);
     store_node<typename P::LF, ODD, T>(f, n3, b, h);
     store_node<typename P::LG, ODD, T>(g, n3, b, k);
 }
@@ -275,14 +339,15 @@ __device__ __forceinline__ void update_node(void* fv, void* gv, const Geometry& 
 template <class P>
 constexpr int kStepMinBlocks = (P::QF + P::QG > 46) ? 2 : (P::QF + P::QG <= 26) ? 4 : LBM_STEP_MINBLOCKS;
 // One AA step for every node of one lattice.
-template <class P, int FORCING, class T, bool ODD>
+template <class P, int FORCING, class T, bool ODD, int LAUNCH>
 __global__ void __launch_bounds__(256, kStepMinBlocks<P>) k_step(StepArgs args)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int x, y;
     const int z = blockIdx.z + args.z0;
-    if (x >= args.geo.nx || y >= args.geo.ny) return;
-    update_node<P, FORCING, T, ODD>(args.f, args.g, args.geo, args.ph, x, y, z);
+    if (!step_unit<LAUNCH>(args, args.geo.nx, x, y, threadIdx.x)) return;
+    wait_prerequisites();
+    update_node<P, FORCING, T, ODD>(args.f, args.g, args.geo, args.ph, x, y, z, [](const float*, const Macro&) {},
+                                    StepPlace<LAUNCH>{args, 1});
 }
 
 // The same step, also reducing the diagnostics (pass 1) of its input state,
@@ -293,17 +358,17 @@ __global__ void __launch_bounds__(256, kStepMinBlocks<P>) k_step(StepArgs args)
 template <class P, int FORCING, class T, bool ODD>
 __global__ void __launch_bounds__(256, 3) k_step_diag(StepArgs args)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int x, y;
     const int z = blockIdx.z;
     constexpr bool kExact = std::is_same<T, float>::value;
     DiagAcc d;
-    if (x < args.geo.nx && y < args.geo.ny) {
+    if (step_unit<kAsked>(args, args.geo.nx, x, y, threadIdx.x)) {
         const uint32_t idx = (uint32_t)x + (uint32_t)args.geo.nx * ((uint32_t)y + (uint32_t)args.geo.ny * (uint32_t)z);
         update_node<P, FORCING, T, ODD>(args.f, args.g, args.geo, args.ph, x, y, z,
                                         [&](const float* h, const Macro& m) {
                                             diag_node<P, kExact>(h, m, args.dg, args.geo.n3, idx, d);
-                                        });
+                                        },
+                                        StepPlace<kAsked>{args, 1});
     }
     const uint32_t blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     d.store_block(args.dg.partials + (size_t)blk * kDNumSlots);
@@ -586,15 +651,16 @@ struct NoHook {
 // One pair's AA update: loads, both collisions (streamed from the words for
 // the plain step; collide_pair_words where a hook reads the nodes' values),
 // stores.
-template <class P, int FORCING, class T, bool ODD, class Hook>
-__device__ __forceinline__ void update_pair(const StepArgs& args, int x0, int y, int z, Hook&& hook)
+template <class P, int FORCING, class T, bool ODD, class Hook, class Place = SamePlace>
+__device__ __forceinline__ void update_pair(const StepArgs& args, int x0, int y, int z, Hook&& hook,
+                                            Place place = Place())
 {
     const uint32_t n3 = args.geo.n3;
     unsigned short* fb = static_cast<unsigned short*>(args.f);
     unsigned short* gb = static_cast<unsigned short*>(args.g);
     uint32_t wf[P::QF], wg[P::QG];
-    const Seam sm(args.geo, x0);
     {
+        const Seam sm(args.geo, x0);
         const PairAddr a(args.geo, x0, y, z);
         load_pair<typename P::LF, ODD>(fb, n3, a, sm, wf);
         load_pair<typename P::LG, ODD>(gb, n3, a, sm, wg);
@@ -605,7 +671,9 @@ __device__ __forceinline__ void update_pair(const StepArgs& args, int x0, int y,
     } else {
         collide_pair_words<P, FORCING, T>(wf, wg, args.ph, hook);
     }
-    const PairAddr b(args.geo, (int)launder(x0), (int)launder(y), (int)launder(z));
+    place(x0, y, z);
+    const Seam sm(args.geo, x0);
+    const PairAddr b(args.geo, x0, y, z);
     store_pair<typename P::LF, ODD>(fb, n3, b, sm, wf);
     store_pair<typename P::LG, ODD>(gb, n3, b, sm, wg);
 }
@@ -616,14 +684,14 @@ __device__ __forceinline__ void update_pair(const StepArgs& args, int x0, int y,
 template <class P>
 constexpr int kStep2MinBlocks = (P::QF + P::QG <= 34) ? 4 : 3;
 
-template <class P, int FORCING, class T, bool ODD>
+template <class P, int FORCING, class T, bool ODD, int LAUNCH>
 __global__ void __launch_bounds__(256, kStep2MinBlocks<P>) k_step2(StepArgs args)
 {
-    const int x0 = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int k, y;
     const int z = blockIdx.z + args.z0;
-    if (x0 >= args.geo.nx || y >= args.geo.ny) return;
-    update_pair<P, FORCING, T, ODD>(args, x0, y, z, NoHook{});
+    if (!step_unit<LAUNCH>(args, args.geo.nx / 2, k, y, threadIdx.x)) return;
+    wait_prerequisites();
+    update_pair<P, FORCING, T, ODD>(args, 2 * k, y, z, NoHook{}, StepPlace<LAUNCH>{args, 2});
 }
 
 // k_step2 that also reduces the diagnostics (pass 1) of its input state, as
@@ -631,18 +699,18 @@ __global__ void __launch_bounds__(256, kStep2MinBlocks<P>) k_step2(StepArgs args
 template <class P, int FORCING, class T, bool ODD>
 __global__ void __launch_bounds__(256, 2) k_step2_diag(StepArgs args)
 {
-    const int x0 = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int k, y;
     const int z = blockIdx.z;
     DiagAcc d;
-    if (x0 < args.geo.nx && y < args.geo.ny) {
+    if (step_unit<kAsked>(args, args.geo.nx / 2, k, y, threadIdx.x)) {
+        const int x0 = 2 * k;
         const uint32_t row = (uint32_t)args.geo.nx * ((uint32_t)y + (uint32_t)args.geo.ny * (uint32_t)z);
         // nodes of the pair's word k = x0 / 2: k and k + half
         const uint32_t lo = row + (uint32_t)(x0 / 2);
         const uint32_t hi = lo + (uint32_t)(args.geo.nx / 2);
         update_pair<P, FORCING, T, ODD>(args, x0, y, z, [&](int which, const float* h, const Macro& m) {
             diag_node<P, false>(h, m, args.dg, args.geo.n3, which ? hi : lo, d);
-        });
+        }, StepPlace<kAsked>{args, 2});
     }
     const uint32_t blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     d.store_block(args.dg.partials + (size_t)blk * kDNumSlots);
