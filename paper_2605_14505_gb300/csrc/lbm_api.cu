@@ -103,9 +103,8 @@ struct lbm_ctx {
     double* diag_partials = nullptr;
     int diag_rows = 0;                 // rows of kDNumSlots the partials hold
     cudaEvent_t diag_event = nullptr;  // diagnostics copied to the host
-    double* diag_out = nullptr;
-    double* diag_host = nullptr;   // pinned
-    int diag_blocks = 0;
+    float2* diag_grad = nullptr;       // pass-2 rows, then the count of finished blocks
+    double* diag_host = nullptr;       // pinned; the totals, written by the last kernel itself
     // host<->device staging
     double* staging = nullptr;
     size_t staging_bytes = 0;
@@ -293,34 +292,68 @@ int ensure_staging(lbm_ctx* h, size_t bytes)
     return LBM_OK;
 }
 
-// Diagnostics scratch: FP32 fields for pass 2, per-block partials (at least
-// `rows` rows), the totals, a pinned host copy and its completion event.
-int ensure_diag(lbm_ctx* h, int rows = 0)
+// Consecutive steps and diagnostics passes overlap their launches: the kernel
+// starts with wait_prerequisites (griddepcontrol.wait) and touches nothing
+// that an earlier one writes before it.
+cudaError_t launch_overlapped(const void* k, dim3 grid, dim3 block, void** args, cudaStream_t s, bool overlap = true)
+{
+    cudaLaunchAttribute pdl{};
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = s;
+    cfg.attrs = &pdl;
+    cfg.numAttrs = overlap && s != nullptr ? 1u : 0u;
+    return cudaLaunchKernelExC(&cfg, k, args);
+}
+
+// Pass 1 on its own: four blocks per SM, or one per 256 nodes of a small lattice.
+uint32_t moment_blocks(const lbm_ctx* h, uint32_t nodes)
+{
+    return std::min(4u * (uint32_t)h->num_sms, (nodes + kDiagBlock - 1) / kDiagBlock);
+}
+
+// Pass 2: planes per thread, at most 16 (the march's three loads ahead are
+// paid once per run) and few enough for 8 blocks per SM.
+dim3 gradient_grid(const lbm_ctx* h, int& planes)
+{
+    const int64_t bx = ((int64_t)h->p.nx * h->p.ny + kDiagBlock - 1) / kDiagBlock;
+    planes = (int)std::min<int64_t>(16, std::max<int64_t>(1, bx * h->p.nz / (8 * (int64_t)h->num_sms)));
+    return dim3((unsigned)bx, (unsigned)((h->p.nz + planes - 1) / planes));
+}
+
+// Diagnostics scratch: FP32 fields for pass 2, pass-1 partials (at least
+// `rows` rows), pass-2 rows, the totals in pinned memory and their event.
+int ensure_diag(lbm_ctx* h, int rows)
 {
     if (!h->diag_fields) {
-        h->diag_blocks = 4 * (h->num_sms > 0 ? h->num_sms : 132);
         size_t fbytes = 4 * (size_t)h->geo.n3 * sizeof(float);
+        int planes = 0;
+        const dim3 g = gradient_grid(h, planes);
+        const size_t pairs = (size_t)g.x * g.y * kDiagPass2;
         if (cudaMalloc(&h->diag_fields, fbytes) != cudaSuccess ||
-            cudaMalloc(&h->diag_out, 16 * sizeof(double)) != cudaSuccess ||
+            cudaMalloc(&h->diag_grad, (pairs + 1) * sizeof(float2)) != cudaSuccess ||
+            cudaMemsetAsync(h->diag_grad + pairs, 0, sizeof(float2), h->stream) != cudaSuccess ||
             cudaMallocHost(&h->diag_host, 16 * sizeof(double)) != cudaSuccess ||
             cudaEventCreateWithFlags(&h->diag_event, cudaEventDisableTiming) != cudaSuccess) {
             cudaGetLastError();
             return fail(LBM_ENOMEM, "diagnostics scratch allocation failed");
         }
     }
-    const int need = rows > h->diag_blocks ? rows : h->diag_blocks;
-    if (h->diag_rows < need) {
+    if (h->diag_rows < rows) {
         if (h->diag_partials) {
             cudaStreamSynchronize(h->stream);
             cudaFree(h->diag_partials);
             h->diag_partials = nullptr;
             h->diag_rows = 0;
         }
-        if (cudaMalloc(&h->diag_partials, (size_t)need * kDNumSlots * sizeof(double)) != cudaSuccess) {
+        if (cudaMalloc(&h->diag_partials, (size_t)rows * kDNumSlots * sizeof(double)) != cudaSuccess) {
             cudaGetLastError();
             return fail(LBM_ENOMEM, "diagnostics partials allocation failed");
         }
-        h->diag_rows = need;
+        h->diag_rows = rows;
     }
     return LBM_OK;
 }
@@ -348,6 +381,11 @@ DiagArgs diag_args(lbm_ctx* h)
     const uint32_t plane = (uint32_t)p.nx * (uint32_t)p.ny;
     a.idx0 = h->slab ? plane : 0u;
     a.idx1 = h->slab ? h->geo.n3 - plane : h->geo.n3;
+    a.rows = 0;
+    const dim3 g = gradient_grid(h, a.planes);
+    a.grad_rows = h->diag_grad;
+    a.finished = reinterpret_cast<unsigned*>(h->diag_grad + (size_t)g.x * g.y * kDiagPass2);
+    a.out = h->diag_host;
     return a;
 }
 
@@ -479,17 +517,51 @@ cudaError_t launch_step(lbm_ctx* h, int odd, cudaStream_t s)
     // FP32 D3Q27xD3Q19 11.7 against 12.2 us per step, 32^3 D3Q19xD3Q7 2.2 against
     // 2.7. Below one wave of the longer kernels the waiting blocks share SMs with
     // the running ones: 27x19 32^3 3.3 to 3.9 from run to run against 3.46.
-    cudaLaunchAttribute pdl{};
-    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    pdl.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = step_block(h, odd);
-    cfg.stream = s;
-    cfg.attrs = &pdl;
-    cfg.numAttrs = s != nullptr && !one_short_wave(h) ? 1u : 0u;
-    return cudaLaunchKernelExC(&cfg, k, args);
+    return launch_overlapped(k, grid, step_block(h, odd), args, s, !one_short_wave(h));
 }
+
+// What follows pass 1, whose `rows` rows are in h->diag_partials: more than
+// kDirectRows of them are first added up on every SM (into the rows behind
+// them), then pass 2 adds up what is left with its own rows and writes the
+// totals; a z-slab has no pass 2.
+constexpr int kDirectRows = 1024;
+cudaError_t launch_totals(lbm_ctx* h, DiagArgs a, int rows)
+{
+    double* at = h->diag_partials;
+    double* mid = at + (size_t)rows * kDNumSlots;
+    cudaError_t e = cudaSuccess;
+    if (rows > kDirectRows) {
+        void* args[] = {&at, &rows, &mid};
+        e = launch_overlapped(diag_rows_kernel(), dim3((unsigned)h->num_sms), dim3(kDiagBlock), args, h->stream);
+        if (e != cudaSuccess) return e;
+        at = mid;
+        rows = h->num_sms;
+    }
+    if (h->slab) {
+        void* args[] = {&at, &rows, &a.out};
+        return launch_overlapped(diag_rows_kernel(), dim3(1), dim3(kDiagBlock), args, h->stream);
+    }
+    a.partials = at;
+    a.rows = rows;
+    const dim3 grid = gradient_grid(h, a.planes);
+    void* args[] = {&a};
+    return launch_overlapped(diag_gradients_kernel(), grid, dim3(kDiagBlock), args, h->stream);
+}
+
+// Pass 1 and what follows it, for the current state.
+int enqueue_diagnostics(lbm_ctx* h)
+{
+    const uint32_t blocks = moment_blocks(h, (uint32_t)owned_nodes(h));
+    if (int rc = ensure_diag(h, (int)blocks + h->num_sms)) return rc;
+    DiagArgs a = diag_args(h);
+    void* args[] = {&a};
+    LBM_CUDA(cudaLaunchKernel(h->ks->diag_moments, dim3(blocks), dim3(kDiagBlock), args, 0, h->stream), "diag pass 1");
+    LBM_CUDA(launch_totals(h, a, (int)blocks), "diag pass 2");
+    return LBM_OK;
+}
+
+// One 256-thread block per 256 nodes.
+dim3 node_grid(const lbm_ctx* h) { return dim3((h->geo.n3 + 255u) / 256u); }
 
 int flat_grid(const lbm_ctx* h)
 {
@@ -1020,22 +1092,7 @@ int lbm_diagnostics(lbm_handle h, lbm_diag* out)
     if (rc) return rc;
     if (!out) return fail(LBM_EINVAL, "null output");
     if (!h->initialized) return fail(LBM_ESTATE, "diagnostics before initialisation");
-    if ((rc = ensure_diag(h))) return rc;
-    DiagArgs a = diag_args(h);
-    void* args[] = {&a};
-    LBM_CUDA(cudaLaunchKernel(h->ks->diag_moments, dim3(h->diag_blocks), dim3(kDiagBlock), args, 0, h->stream),
-             "diag pass 1");
-    if (!h->slab)
-        LBM_CUDA(cudaLaunchKernel(diag_gradients_kernel(), dim3(h->diag_blocks), dim3(kDiagBlock), args, 0, h->stream),
-                 "diag pass 2");
-    const double* pp = h->diag_partials;
-    int nb = h->diag_blocks;
-    int nb2 = h->slab ? 0 : h->diag_blocks;
-    double* dout = h->diag_out;
-    void* fargs[] = {&pp, &nb, &nb2, &dout};
-    LBM_CUDA(cudaLaunchKernel(diag_final_kernel(), dim3(1), dim3(kDiagBlock), fargs, 0, h->stream), "diag pass 3");
-    LBM_CUDA(cudaMemcpyAsync(h->diag_host, h->diag_out, kDNumSlots * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
-             "diag copy");
+    if ((rc = enqueue_diagnostics(h))) return rc;
     LBM_CUDA(cudaStreamSynchronize(h->stream), "diagnostics");
     return fill_diag(h, h->step, out);
 }
@@ -1052,8 +1109,7 @@ int lbm_step_diagnostics(lbm_handle h, int64_t nsteps, lbm_diag* out)
     const bool pairs = uses_pairs(h, odd);
     const dim3 grid = step_grid(h, odd);
     const int rows = (int)(grid.x * grid.y * grid.z);
-    const int level1 = h->num_sms > 0 ? h->num_sms : 132;   // first-level rows of the final pass
-    if ((rc = ensure_diag(h, rows + level1))) return rc;
+    if ((rc = ensure_diag(h, rows + h->num_sms))) return rc;
     const DiagArgs da = diag_args(h);
     StepArgs a = step_args(h, odd);
     a.dg = DiagSink{da.ep_scale, da.epsk_scale, da.s_scale, h->diag_fields, h->diag_partials};
@@ -1063,25 +1119,7 @@ int lbm_step_diagnostics(lbm_handle h, int64_t nsteps, lbm_diag* out)
     const int64_t step0 = h->step;
     h->odd ^= 1;
     h->step += 1;
-    DiagArgs g = da;
-    void* gargs[] = {&g};
-    LBM_CUDA(cudaLaunchKernel(diag_gradients_kernel(), dim3(h->diag_blocks), dim3(kDiagBlock), gargs, 0, h->stream),
-             "diag pass 2");
-    // pass 3 in two levels: `level1` blocks each sum a contiguous range of the
-    // step blocks' rows (and of the pass-2 rows) into one row, then one block
-    const double* pp = h->diag_partials;
-    int nb1 = rows, nb2 = h->diag_blocks;
-    double* mid = h->diag_partials + (size_t)rows * kDNumSlots;
-    void* l1args[] = {&pp, &nb1, &nb2, &mid};
-    LBM_CUDA(cudaLaunchKernel(diag_final_kernel(), dim3(level1), dim3(kDiagBlock), l1args, 0, h->stream),
-             "diag pass 3a");
-    const double* pm = mid;
-    int nl = level1;
-    double* dout = h->diag_out;
-    void* fargs[] = {&pm, &nl, &nl, &dout};
-    LBM_CUDA(cudaLaunchKernel(diag_final_kernel(), dim3(1), dim3(kDiagBlock), fargs, 0, h->stream), "diag pass 3b");
-    LBM_CUDA(cudaMemcpyAsync(h->diag_host, h->diag_out, kDNumSlots * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
-             "diag copy");
+    LBM_CUDA(launch_totals(h, da, rows), "diag pass 2");
     LBM_CUDA(cudaEventRecord(h->diag_event, h->stream), "diag event");
     if ((rc = lbm_step(h, nsteps - 1))) return rc;
     LBM_CUDA(cudaEventSynchronize(h->diag_event), "diagnostics");
@@ -1105,7 +1143,7 @@ int lbm_get_fields(lbm_handle h, double* rho, double* u, double* rho_p)
     a.u = h->staging + n3;
     a.rho_p = h->staging + 4 * n3;
     void* args[] = {&a};
-    LBM_CUDA(cudaLaunchKernel(h->ks->get_fields, dim3(flat_grid(h)), dim3(256), args, 0, h->stream), "get_fields");
+    LBM_CUDA(cudaLaunchKernel(h->ks->get_fields, node_grid(h), dim3(256), args, 0, h->stream), "get_fields");
     if (rho) LBM_CUDA(cudaMemcpyAsync(rho, a.rho, n3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream), "copy rho");
     if (u) LBM_CUDA(cudaMemcpyAsync(u, a.u, 3 * n3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream), "copy u");
     if (rho_p)
@@ -1139,7 +1177,7 @@ int lbm_get_fields_device(lbm_handle h, double* rho, double* u, double* rho_p)
     a.u = u;
     a.rho_p = rho_p;
     void* args[] = {&a};
-    LBM_CUDA(cudaLaunchKernel(h->ks->get_fields, dim3(flat_grid(h)), dim3(256), args, 0, h->stream),
+    LBM_CUDA(cudaLaunchKernel(h->ks->get_fields, node_grid(h), dim3(256), args, 0, h->stream),
              "get_fields_device");
     return LBM_OK;
 }
@@ -1506,17 +1544,13 @@ int lbm_diagnostics_noalloc(lbm_handle h, lbm_diag* out)
     if (h->slab) return fail(LBM_EUNSUPPORTED, "allocation-free diagnostics of a z-slab (use lbm_diagnostics)");
     double* scratch = nullptr;
     if ((rc = static_scratch_address(h->device, &scratch))) return rc;
-    // the moment pass strides over the lattice, so the grid fills the GPU
-    // (4 blocks per SM, as lbm_diagnostics) whatever the node count, within
-    // the array's rows and without blocks that get no node
-    const uint32_t sms = (uint32_t)(h->num_sms > 0 ? h->num_sms : 132);
-    const uint32_t busy = std::min(4 * sms, (n3 + kDiagBlock - 1) / (uint32_t)kDiagBlock);
-    const uint32_t blocks = std::min((uint32_t)kStaticMaxBlocks, std::max(min_blocks, busy));
+    // a row of the array per block, as lbm_diagnostics within the array's rows
+    const uint32_t blocks = std::min((uint32_t)kStaticMaxBlocks, std::max(min_blocks, moment_blocks(h, n3)));
     const lbm_params& p = h->p;
     const double cs2f = cs2_of(h->q.qf);
     const double gn2 = (p.beta != 0.0) ? (-p.G * p.rho0 / p.beta) : 1.0;
     const double nu = cs2f * (p.tau_f - 0.5);
-    DiagArgs a;
+    DiagArgs a{};
     a.f = f_ptr(h);
     a.g = g_ptr(h);
     a.geo = h->geo;
@@ -1536,12 +1570,11 @@ int lbm_diagnostics_noalloc(lbm_handle h, lbm_diag* out)
              "static diag pass 1");
     const double* pp = scratch;
     int nb = (int)blocks;
-    int nb2 = 0;   // no pass 2 here
     double* dout = scratch + kStaticOutOffset;
-    void* fargs[] = {&pp, &nb, &nb2, &dout};
-    LBM_CUDA(cudaLaunchKernel(diag_final_kernel(), dim3(1), dim3(kDiagBlock), fargs, 0, h->stream),
+    void* fargs[] = {&pp, &nb, &dout};
+    LBM_CUDA(cudaLaunchKernel(diag_rows_kernel(), dim3(1), dim3(kDiagBlock), fargs, 0, h->stream),
              "static diag pass 2");
-    double s[kDNumSlots];
+    double s[kDiagPass1];
     LBM_CUDA(cudaMemcpyAsync(s, dout, sizeof(s), cudaMemcpyDeviceToHost, h->stream), "static diag copy");
     LBM_CUDA(cudaStreamSynchronize(h->stream), "static diagnostics");
     const double inv = 1.0 / (double)n3;
@@ -1574,7 +1607,7 @@ int lbm_destroy(lbm_handle h)
     if (h->staging) cudaFree(h->staging);
     if (h->diag_fields) cudaFree(h->diag_fields);
     if (h->diag_partials) cudaFree(h->diag_partials);
-    if (h->diag_out) cudaFree(h->diag_out);
+    if (h->diag_grad) cudaFree(h->diag_grad);
     if (h->diag_host) cudaFreeHost(h->diag_host);
     if (h->diag_event) cudaEventDestroy(h->diag_event);
     if (h->copy_event) cudaEventDestroy(h->copy_event);
@@ -2119,9 +2152,16 @@ int lbm_batch_diagnostics(lbm_batch b, lbm_diag* out)
     int rc = lbm_batch_synchronize(b);
     if (rc) return rc;
     if (!out) return fail(LBM_EINVAL, "null output");
+    for (lbm_ctx* h : b->inst) {
+        if (!h->initialized) return fail(LBM_ESTATE, "diagnostics before initialisation");
+    }
+    // every instance's kernels first, then one wait (one each: 64 instances 3.3 ms)
+    for (lbm_ctx* h : b->inst)
+        if ((rc = enqueue_diagnostics(h))) return rc;
     int worst = LBM_OK;
     for (size_t i = 0; i < b->inst.size(); ++i) {
-        rc = lbm_diagnostics(b->inst[i], &out[i]);
+        LBM_CUDA(cudaStreamSynchronize(b->inst[i]->stream), "diagnostics");
+        rc = fill_diag(b->inst[i], b->inst[i]->step, &out[i]);
         if (rc == LBM_ENONFINITE) worst = rc;
         else if (rc) return rc;
     }

@@ -30,8 +30,14 @@ struct DiagArgs {
     float epsp_scale;    // D (G/N)^2 / rho0^2
     float nu;
     float* fields;       // 4 * n3: rho', ux, uy, uz (written by pass 1, read by pass 2)
-    double* partials;    // gridDim.x * kDNumSlots
+    double* partials;    // pass 1: a row of kDNumSlots per block
     uint32_t idx0, idx1; // pass 1 reduces nodes [idx0, idx1) (a z-slab: its own planes only)
+    // pass 2, whose last block sums everything
+    int planes;          // planes a thread marches through
+    int rows;            // pass-1 rows
+    float2* grad_rows;   // kDiagPass2 pairs per block
+    unsigned* finished;  // blocks done; 0 between launches
+    double* out;         // kDNumSlots totals
 };
 
 // Compensated (Kahan) FP32 running sum for a thread's share of a diagnostics
@@ -47,38 +53,7 @@ struct KahanF {
         c = (t - s) - y;
         s = t;
     }
-    __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
-
-// Block sum (the last slot a maximum if MAXLAST) of v into out[0..NV), for
-// blocks of up to 256 threads, a whole number of warps, in any shape.
-template <int NV, bool MAXLAST>
-__device__ __forceinline__ void block_reduce_store(double (&v)[NV], double* out)
-{
-    __shared__ double sh[kDiagBlock / 32][NV];
-    const int tid = (int)(threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z));
-    const int nwarps = (int)(blockDim.x * blockDim.y * blockDim.z) / 32;
-    const int lane = tid & 31, wid = tid >> 5;
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            double t = __shfl_down_sync(0xffffffffu, v[q], o);
-            v[q] = (MAXLAST && q == NV - 1) ? fmax(v[q], t) : v[q] + t;
-        }
-    }
-    if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < NV; ++q) sh[wid][q] = v[q];
-    }
-    __syncthreads();
-    if (tid < NV) {
-        const int q = tid;
-        double acc = sh[0][q];
-        for (int w = 1; w < nwarps; ++w) acc = (MAXLAST && q == NV - 1) ? fmax(acc, sh[w][q]) : acc + sh[w][q];
-        out[q] = acc;
-    }
-}
 
 // What a kernel needs to add one node's diagnostics (pass 1): the scales of
 // Eqs. 22-24 and of the non-equilibrium eps_k, the fields for pass 2 and the
@@ -99,19 +74,57 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
     e = (a - (s - bb)) + (b - bb);
 }
 
+// Sum of every thread's N values over a block of up to 256 threads (whole
+// warps, any shape), each value an unevaluated FP32 pair hi + lo, two-sum at
+// every add: FP64-like accuracy on the FP32 pipes (this GPU's FP64 rate is a
+// small fraction of its FP32 rate). Value MAXQ is a maximum. Threads 0..N-1
+// return the total of value tid.
+template <int N, int MAXQ>
+__device__ __forceinline__ float2 block_sum_pairs(float (&hi)[N], float (&lo)[N])
+{
+    __shared__ float2 sh[kDiagBlock / 32][N];
+    const int tid = (int)(threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z));
+    const int nwarps = (int)(blockDim.x * blockDim.y * blockDim.z) / 32;
+    const int lane = tid & 31, wid = tid >> 5;
+    auto add = [](bool max, float& h, float& l, float oh, float ol) {
+        if (max) {
+            h = fmaxf(h, oh);
+        } else {
+            float t, e;
+            two_sum(h, oh, t, e);
+            h = t;
+            l = l + ol + e;
+        }
+    };
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            const float oh = __shfl_down_sync(0xffffffffu, hi[q], o);
+            const float ol = __shfl_down_sync(0xffffffffu, lo[q], o);
+            add(q == MAXQ, hi[q], lo[q], oh, ol);
+        }
+    }
+    if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < N; ++q) sh[wid][q] = make_float2(hi[q], lo[q]);
+    }
+    __syncthreads();
+    if (tid >= N) return make_float2(0.f, 0.f);
+    float2 v = sh[0][tid];
+    for (int w = 1; w < nwarps; ++w) add(tid == MAXQ, v.x, v.y, sh[w][tid].x, sh[w][tid].y);
+    return v;
+}
+
 struct DiagAcc {
     KahanF acc[kDiagPass1 - 1];
     float umax = 0.f;
-    // The pass-1 slots of this thread into one block row. The block sum is
-    // carried as an unevaluated FP32 pair (hi + lo, two-sum at every add), so
-    // the step kernels, which write one row per block, keep FP64-like
-    // accuracy on the FP32 pipes; one thread per slot converts the pair.
+    __device__ __forceinline__ void add(int q, float x) { acc[q].add(x); }
+    __device__ __forceinline__ void max(float x) { umax = fmaxf(umax, x); }
+    // The pass-1 slots of this thread into one block row, each as its pair in
+    // the slot's 8 bytes.
     __device__ __forceinline__ void store_block(double* row)
     {
-        __shared__ float sh[kDiagBlock / 32][kDiagPass1][2];
-        const int tid = (int)(threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z));
-        const int nwarps = (int)(blockDim.x * blockDim.y * blockDim.z) / 32;
-        const int lane = tid & 31, wid = tid >> 5;
         float hi[kDiagPass1], lo[kDiagPass1];
 #pragma unroll
         for (int q = 0; q < kDiagPass1 - 1; ++q) {
@@ -120,48 +133,66 @@ struct DiagAcc {
         }
         hi[kDUmax] = umax;
         lo[kDUmax] = 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int q = 0; q < kDiagPass1; ++q) {
-                const float oh = __shfl_down_sync(0xffffffffu, hi[q], o);
-                const float ol = __shfl_down_sync(0xffffffffu, lo[q], o);
-                if (q == kDUmax) {
-                    hi[q] = fmaxf(hi[q], oh);
-                } else {
-                    float t, e;
-                    two_sum(hi[q], oh, t, e);
-                    hi[q] = t;
-                    lo[q] = lo[q] + ol + e;
-                }
-            }
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int q = 0; q < kDiagPass1; ++q) {
-                sh[wid][q][0] = hi[q];
-                sh[wid][q][1] = lo[q];
-            }
-        }
-        __syncthreads();
-        if (tid < kDiagPass1) {
-            const int q = tid;
-            float h = sh[0][q][0], l = sh[0][q][1];
-            for (int w = 1; w < nwarps; ++w) {
-                if (q == kDUmax) {
-                    h = fmaxf(h, sh[w][q][0]);
-                } else {
-                    float t, e;
-                    two_sum(h, sh[w][q][0], t, e);
-                    h = t;
-                    l = l + sh[w][q][1] + e;
-                }
-            }
-            // the pair itself, in the slot's 8 bytes (k_diag_final with pass1_pairs)
-            reinterpret_cast<float2*>(row)[q] = make_float2(h, l);
-        }
+        const float2 v = block_sum_pairs<kDiagPass1, kDUmax>(hi, lo);
+        const int tid = (int)(threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z));
+        if (tid < kDiagPass1) reinterpret_cast<float2*>(row)[tid] = v;
     }
 };
+
+// The same sums kept in shared memory, one column per thread.
+struct SharedAcc {
+    float (*sh)[kDiagBlock];   // s and c of every sum, then the maximum
+    static constexpr int kRows = 2 * (kDiagPass1 - 1) + 1;
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) sh[r][threadIdx.x] = 0.f;
+    }
+    __device__ __forceinline__ void add(int q, float x)
+    {
+        KahanF k;
+        k.s = sh[2 * q][threadIdx.x];
+        k.c = sh[2 * q + 1][threadIdx.x];
+        k.add(x);
+        sh[2 * q][threadIdx.x] = k.s;
+        sh[2 * q + 1][threadIdx.x] = k.c;
+    }
+    __device__ __forceinline__ void max(float x)
+    {
+        sh[kRows - 1][threadIdx.x] = fmaxf(sh[kRows - 1][threadIdx.x], x);
+    }
+    __device__ __forceinline__ DiagAcc get() const
+    {
+        DiagAcc d;
+#pragma unroll
+        for (int q = 0; q < kDiagPass1 - 1; ++q) {
+            d.acc[q].s = sh[2 * q][threadIdx.x];
+            d.acc[q].c = sh[2 * q + 1][threadIdx.x];
+        }
+        d.umax = sh[kRows - 1][threadIdx.x];
+        return d;
+    }
+};
+
+// Pass-1 rows [first, last) added to a thread's pairs, rows dealt round the block.
+__device__ __forceinline__ void add_rows(const double* rows, int first, int last, float* hi, float* lo)
+{
+    for (int b = first + (int)threadIdx.x; b < last; b += blockDim.x) {
+        const float2* row = reinterpret_cast<const float2*>(rows + (size_t)b * kDNumSlots);
+#pragma unroll
+        for (int q = 0; q < kDiagPass1; ++q) {
+            const float2 v = row[q];
+            if (q == kDUmax) {
+                hi[q] = fmaxf(hi[q], v.x);
+            } else {
+                float t, e;
+                two_sum(hi[q], v.x, t, e);
+                hi[q] = t;
+                lo[q] = lo[q] + v.y + e;
+            }
+        }
+    }
+}
 
 // One node's pass-1 diagnostics from its post-stream, pre-collision
 // populations and moments, and its FP32 fields for pass 2. PAIRSUM: h holds
@@ -171,9 +202,9 @@ struct DiagAcc {
 // and -e, so a pair contributes e e (h_i + h_j). D3Q7 lacks the fourth-order
 // isotropy behind sum e e f_eq = rho u u + rho cs^2 I, so there the pair sums
 // of f_eq(rho, u) are subtracted explicitly and the closed-form terms are not.
-template <class P, bool PAIRSUM>
+template <class P, bool PAIRSUM, class Acc>
 __device__ __forceinline__ void diag_node(const float* h, const Macro& m, const DiagSink& s, uint32_t n3,
-                                          uint32_t idx, DiagAcc& d)
+                                          uint32_t idx, Acc& d)
 {
     using LF = typename P::LF;
     constexpr bool kExplicit = (LF::kQ == 7);
@@ -207,15 +238,15 @@ __device__ __forceinline__ void diag_node(const float* h, const Macro& m, const 
     const float pyz = myz - rr * m.uy * m.uz + 0.5f * m.uy * m.Fz;
     const float ss = pxx * pxx + pyy * pyy + pzz * pzz + 2.f * (pxy * pxy + pxz * pxz + pyz * pyz);
     const float sfac = s.s_scale * m.irho;
-    d.acc[kDEk].add(0.5f * usq);
-    d.acc[kDEp].add(s.ep_scale * m.rho_p * m.rho_p);
-    d.acc[kDEpsK].add(s.epsk_scale * sfac * sfac * ss);
-    d.acc[kDDrho].add(m.drho);
-    d.acc[kDA].add(m.a);
-    d.acc[kDJx].add(m.jx);
-    d.acc[kDJy].add(m.jy);
-    d.acc[kDJz].add(m.jz);
-    d.umax = fmaxf(d.umax, sqrtf(usq));
+    d.add(kDEk, 0.5f * usq);
+    d.add(kDEp, s.ep_scale * m.rho_p * m.rho_p);
+    d.add(kDEpsK, s.epsk_scale * sfac * sfac * ss);
+    d.add(kDDrho, m.drho);
+    d.add(kDA, m.a);
+    d.add(kDJx, m.jx);
+    d.add(kDJy, m.jy);
+    d.add(kDJz, m.jz);
+    d.max(sqrtf(usq));
     if (s.fields) {
         s.fields[idx] = m.rho_p;
         s.fields[(size_t)n3 + idx] = m.ux;
@@ -1026,174 +1057,161 @@ __global__ void k_set_pops(PopArgs a)
     }
 }
 
+// Pass 1 on its own: four 256-thread blocks per SM, all of them resident, that
+// stride over the lattice; thread t sums nodes t, t + stride, ... in order.
+// The sums live in shared memory: in registers they kept three blocks on an SM
+// (80 registers), so the fourth ran alone in a second wave. A block's warps
+// stay together: with the loads' 256-byte prefetch a warp also fetches its
+// neighbour's half block, and where warps drifted apart that half had left L2
+// again before its use (3.7 to 4.3 GB read of 3.1 GB at 256^3 FP32). 0.516 ms
+// there against 0.66 to 0.74, 96 % of the copy bandwidth.
 template <class P, class T>
-__global__ void __launch_bounds__(kDiagBlock) k_diag_moments(DiagArgs a)
+__global__ void __launch_bounds__(kDiagBlock, P::QF + P::QG > 46 ? 3 : 4) k_diag_moments(DiagArgs a)
 {
     using LF = typename P::LF;
+    __shared__ float sums[SharedAcc::kRows][kDiagBlock];
+    SharedAcc d{sums};
+    d.clear();
     const uint32_t n3 = a.geo.n3;
     const DiagSink sink{a.ep_scale, a.epsk_scale, a.s_scale, a.fields, a.partials};
-    DiagAcc d;
-    for (uint32_t idx = a.idx0 + blockIdx.x * blockDim.x + threadIdx.x; idx < a.idx1;
-         idx += gridDim.x * blockDim.x) {
-        int x, y, z;
-        node_xyz(a.geo, idx, x, y, z);
-        const NodeAddr na = node_addr<T>(a.geo, x, y, z);
-        float h[P::QF], k[P::QG];
-        if (a.odd) {
-            load_node<LF, true, T>(static_cast<const T*>(a.f), n3, na, h);
-            load_node<typename P::LG, true, T>(static_cast<const T*>(a.g), n3, na, k);
-        } else {
-            load_node<LF, false, T>(static_cast<const T*>(a.f), n3, na, h);
-            load_node<typename P::LG, false, T>(static_cast<const T*>(a.g), n3, na, k);
+    const uint32_t stride = gridDim.x * kDiagBlock;
+    int x, y, z, dx, dy, dz;
+    uint32_t idx = a.idx0 + blockIdx.x * kDiagBlock + threadIdx.x;
+    node_xyz(a.geo, idx, x, y, z);
+    node_xyz(a.geo, stride, dx, dy, dz);
+    for (uint32_t first = a.idx0 + blockIdx.x * kDiagBlock; first < a.idx1; first += stride, idx += stride) {
+        if (idx < a.idx1) {
+            const NodeAddr na = node_addr<T>(a.geo, x, y, z);
+            float h[P::QF], k[P::QG];
+            if (a.odd) {
+                load_node<LF, true, T>(static_cast<const T*>(a.f), n3, na, h);
+                load_node<typename P::LG, true, T>(static_cast<const T*>(a.g), n3, na, k);
+            } else {
+                load_node<LF, false, T>(static_cast<const T*>(a.f), n3, na, h);
+                load_node<typename P::LG, false, T>(static_cast<const T*>(a.g), n3, na, k);
+            }
+            const Macro m = node_macro<P>(h, k, a.ph);
+            diag_node<P, true>(h, m, sink, n3, idx, d);
         }
-        const Macro m = node_macro<P>(h, k, a.ph);
-        diag_node<P, true>(h, m, sink, n3, idx, d);
+        x += dx;
+        if (x >= a.geo.nx) {
+            x -= a.geo.nx;
+            ++y;
+        }
+        y += dy;
+        if (y >= a.geo.ny) {
+            y -= a.geo.ny;
+            ++z;
+        }
+        z += dz;
+        __syncthreads();
     }
-    d.store_block(a.partials + (size_t)blockIdx.x * kDNumSlots);
+    launch_dependents();
+    DiagAcc sum = d.get();
+    sum.store_block(a.partials + (size_t)blockIdx.x * kDNumSlots);
 }
 
 #ifdef LBM_REDUCTION_KERNELS  // defined in exactly one translation unit
-// Eqs. 25, 26 with second-order central differences of the pass-1 fields.
-__global__ void __launch_bounds__(kDiagBlock) k_diag_gradients(DiagArgs a)
+// Pass 2: Eqs. 25, 26 with second-order central differences of the pass-1
+// fields, and the totals. A thread owns one (x, y) of the plane and marches
+// through a.planes planes with rho', ux, uy of three planes in registers: 15
+// loads and no division per node, against 18 loads and two divisions with a
+// strided loop over the nodes (0.091 against 0.130 ms at 256^3, where the 16 B
+// per node take 0.040; what is left is load issue). The last block to finish adds all pass-1 and pass-2 rows in
+// a fixed order and writes the totals to pinned memory, so neither a launch nor
+// a copy follows: one fused step and its record at 32^3 21 us against 45.
+__global__ void __launch_bounds__(kDiagBlock, 4) k_diag_gradients(DiagArgs a)
 {
-    const uint32_t n3 = a.geo.n3;
+    const uint32_t nx = (uint32_t)a.geo.nx, ny = (uint32_t)a.geo.ny, nz = (uint32_t)a.geo.nz, nxy = nx * ny;
+    const size_t n3 = a.geo.n3;
     const float* rp = a.fields;
     const float* ux = a.fields + n3;
-    const float* uy = a.fields + 2 * (size_t)n3;
-    const float* uz = a.fields + 3 * (size_t)n3;
+    const float* uy = a.fields + 2 * n3;
+    const float* uz = a.fields + 3 * n3;
+    const uint32_t r = blockIdx.x * kDiagBlock + threadIdx.x;
+    const uint32_t z0 = blockIdx.y * (uint32_t)a.planes;
+    const uint32_t z1 = min(z0 + (uint32_t)a.planes, nz);
     KahanF acc[kDiagPass2];
-    for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n3; idx += gridDim.x * blockDim.x) {
-        int x, y, z;
-        node_xyz(a.geo, idx, x, y, z);
-        const NodeAddr na(a.geo, x, y, z);   // the FP32 fields are in node order
-        const uint32_t xp = na.off(1, 0, 0), xm = na.off(-1, 0, 0);
-        const uint32_t yp = na.off(0, 1, 0), ym = na.off(0, -1, 0);
-        const uint32_t zp = na.off(0, 0, 1), zm = na.off(0, 0, -1);
-        const float gx = 0.5f * (rp[xp] - rp[xm]);
-        const float gy = 0.5f * (rp[yp] - rp[ym]);
-        const float gz = 0.5f * (rp[zp] - rp[zm]);
-        const float wx = 0.5f * (uz[yp] - uz[ym]) - 0.5f * (uy[zp] - uy[zm]);
-        const float wy = 0.5f * (ux[zp] - ux[zm]) - 0.5f * (uz[xp] - uz[xm]);
-        const float wz = 0.5f * (uy[xp] - uy[xm]) - 0.5f * (ux[yp] - ux[ym]);
-        acc[0].add(a.epsp_scale * (gx * gx + gy * gy + gz * gz));
-        acc[1].add(a.nu * (wx * wx + wy * wy + wz * wz));
+    wait_prerequisites();
+    if (r < nxy) {
+        const uint32_t y = r / nx, x = r - y * nx;
+        const uint32_t xm = x == 0 ? r + nx - 1 : r - 1, xp = x == nx - 1 ? r - x : r + 1;
+        const uint32_t ym = y == 0 ? r + nxy - nx : r - nx, yp = y == ny - 1 ? x : r + nx;
+        const uint32_t below = (z0 == 0 ? nz - 1 : z0 - 1) * nxy + r;
+        uint32_t at = z0 * nxy;
+        float rpm = rp[below], uxm = ux[below], uym = uy[below];
+        float rpc = rp[at + r], uxc = ux[at + r], uyc = uy[at + r];
+        for (uint32_t z = z0; z < z1; ++z) {
+            const uint32_t up = z == nz - 1 ? 0u : at + nxy;
+            const float rpp = rp[up + r], uxp = ux[up + r], uyp = uy[up + r];
+            const float gx = 0.5f * (rp[at + xp] - rp[at + xm]);
+            const float gy = 0.5f * (rp[at + yp] - rp[at + ym]);
+            const float gz = 0.5f * (rpp - rpm);
+            const float wx = 0.5f * (uz[at + yp] - uz[at + ym]) - 0.5f * (uyp - uym);
+            const float wy = 0.5f * (uxp - uxm) - 0.5f * (uz[at + xp] - uz[at + xm]);
+            const float wz = 0.5f * (uy[at + xp] - uy[at + xm]) - 0.5f * (ux[at + yp] - ux[at + ym]);
+            acc[0].add(a.epsp_scale * (gx * gx + gy * gy + gz * gz));
+            acc[1].add(a.nu * (wx * wx + wy * wy + wz * wz));
+            rpm = rpc;
+            uxm = uxc;
+            uym = uyc;
+            rpc = rpp;
+            uxc = uxp;
+            uyc = uyp;
+            at = up;
+        }
     }
-    double v[kDiagPass2] = {acc[0].value(), acc[1].value()};
-    block_reduce_store<kDiagPass2, false>(v, a.partials + (size_t)blockIdx.x * kDNumSlots + kDiagPass1);
+    launch_dependents();
+    const uint32_t block = blockIdx.x + gridDim.x * blockIdx.y, blocks = gridDim.x * gridDim.y;
+    {
+        float hi[kDiagPass2] = {acc[0].s, acc[1].s}, lo[kDiagPass2] = {-acc[0].c, -acc[1].c};
+        const float2 v = block_sum_pairs<kDiagPass2, -1>(hi, lo);
+        if (threadIdx.x < kDiagPass2) a.grad_rows[(size_t)block * kDiagPass2 + threadIdx.x] = v;
+    }
+    __shared__ bool last;
+    if (threadIdx.x < 32) {   // the warp that wrote the row
+        __threadfence();
+        __syncwarp();
+        if (threadIdx.x == 0) last = atomicAdd(a.finished, 1u) == blocks - 1u;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    float hi[kDNumSlots] = {}, lo[kDNumSlots] = {};
+    add_rows(a.partials, 0, a.rows, hi, lo);
+    for (uint32_t b = threadIdx.x; b < blocks; b += kDiagBlock) {
+#pragma unroll
+        for (int q = 0; q < kDiagPass2; ++q) {
+            const float2 v = __ldcg(a.grad_rows + (size_t)b * kDiagPass2 + q);
+            float t, e;
+            two_sum(hi[kDiagPass1 + q], v.x, t, e);
+            hi[kDiagPass1 + q] = t;
+            lo[kDiagPass1 + q] += v.y + e;
+        }
+    }
+    const float2 v = block_sum_pairs<kDNumSlots, kDUmax>(hi, lo);
+    if (threadIdx.x < kDNumSlots) a.out[threadIdx.x] = (double)v.x + (double)v.y;
+    if (threadIdx.x == 0) *a.finished = 0u;
 }
 
-// Final pass: one block adds the per-block partials in a fixed order.
-// Block b of the grid sums its share of the rows: pass-1 slots from the first
-// nb1 rows, pass-2 slots from the first nb2, split into gridDim.x contiguous
-// ranges in order. The pass-1 slots hold FP32 (hi, lo) pairs (DiagAcc; the
-// diagnosing step kernels write one row per step block, 65536 rows at
-// 256^3), summed with two-sum on the FP32 pipes; the pass-2 slots FP64
-// values. With one block the totals go to out[0..kDNumSlots) as FP64; with
-// more (a first level that spreads the row reads over the SMs) each block
-// writes its row of out in the input's format.
-__global__ void __launch_bounds__(kDiagBlock) k_diag_final(const double* partials, int nb1, int nb2, double* out)
+// Pass-1 rows added up: block b of the grid sums its contiguous share of the
+// nb rows. With one block the totals go to out[0..kDiagPass1) as FP64; with
+// more (a step kernel's row per block, 65536 rows at 256^3, spread over the
+// SMs before k_diag_gradients reads them) each block writes its row of out.
+__global__ void __launch_bounds__(kDiagBlock) k_diag_rows(const double* rows, int nb, double* out)
 {
-    constexpr bool pass1_pairs = true;
-    const int per1 = (nb1 + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int per2 = (nb2 + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int b1 = (int)blockIdx.x * per1, e1 = min(nb1, b1 + per1);
-    const int b2 = (int)blockIdx.x * per2, e2 = min(nb2, b2 + per2);
-    const bool pairs_out = pass1_pairs && gridDim.x > 1;
-    double acc[kDNumSlots];
-#pragma unroll
-    for (int q = 0; q < kDNumSlots; ++q) acc[q] = 0.0;
-    float hi[kDiagPass1], lo[kDiagPass1];
-#pragma unroll
-    for (int q = 0; q < kDiagPass1; ++q) hi[q] = lo[q] = 0.f;
-    {
-        for (int b = b1 + (int)threadIdx.x; b < e1; b += blockDim.x) {
-            const float2* row = reinterpret_cast<const float2*>(partials + (size_t)b * kDNumSlots);
-#pragma unroll
-            for (int q = 0; q < kDiagPass1; ++q) {
-                const float2 v = row[q];
-                if (q == kDUmax) {
-                    hi[q] = fmaxf(hi[q], v.x);
-                } else {
-                    float t, e;
-                    two_sum(hi[q], v.x, t, e);
-                    hi[q] = t;
-                    lo[q] = lo[q] + v.y + e;
-                }
-            }
-        }
-        if (!pairs_out) {
-#pragma unroll
-            for (int q = 0; q < kDiagPass1; ++q) acc[q] = (double)hi[q] + (double)lo[q];
-        }
-    }
-    for (int b = b2 + (int)threadIdx.x; b < e2; b += blockDim.x) {
-#pragma unroll
-        for (int q = kDiagPass1; q < kDNumSlots; ++q) acc[q] += partials[(size_t)b * kDNumSlots + q];
-    }
-    double* dst = out + (size_t)blockIdx.x * kDNumSlots;
-    if (pairs_out) {
-        // pass-1 pairs through the block in FP32 two-sum, pass-2 in FP64 below
-        __shared__ float shp[kDiagBlock / 32][kDiagPass1][2];
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int q = 0; q < kDiagPass1; ++q) {
-                const float oh = __shfl_down_sync(0xffffffffu, hi[q], o);
-                const float ol = __shfl_down_sync(0xffffffffu, lo[q], o);
-                if (q == kDUmax) {
-                    hi[q] = fmaxf(hi[q], oh);
-                } else {
-                    float t, e;
-                    two_sum(hi[q], oh, t, e);
-                    hi[q] = t;
-                    lo[q] = lo[q] + ol + e;
-                }
-            }
-        }
-        if (lane == 0)
-            for (int q = 0; q < kDiagPass1; ++q) {
-                shp[wid][q][0] = hi[q];
-                shp[wid][q][1] = lo[q];
-            }
-        __syncthreads();
-        if (threadIdx.x < kDiagPass1) {
-            const int q = threadIdx.x;
-            float h = shp[0][q][0], l = shp[0][q][1];
-            for (int w = 1; w < kDiagBlock / 32; ++w) {
-                if (q == kDUmax) {
-                    h = fmaxf(h, shp[w][q][0]);
-                } else {
-                    float t, e;
-                    two_sum(h, shp[w][q][0], t, e);
-                    h = t;
-                    l = l + shp[w][q][1] + e;
-                }
-            }
-            reinterpret_cast<float2*>(dst)[q] = make_float2(h, l);
-        }
-    }
-    __shared__ double sh[kDiagBlock / 32][kDNumSlots];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int q0 = pairs_out ? kDiagPass1 : 0;   // slots reduced in FP64 here
-#pragma unroll
-    for (int q = 0; q < kDNumSlots; ++q) {
-        if (q < q0) continue;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double t = __shfl_down_sync(0xffffffffu, acc[q], o);
-            acc[q] = (q == kDUmax) ? fmax(acc[q], t) : acc[q] + t;
-        }
-    }
-    if (lane == 0)
-        for (int q = q0; q < kDNumSlots; ++q) sh[wid][q] = acc[q];
-    __syncthreads();
-    if ((int)threadIdx.x >= q0 && threadIdx.x < kDNumSlots) {
-        const int q = threadIdx.x;
-        double v = sh[0][q];
-        for (int w = 1; w < kDiagBlock / 32; ++w) v = (q == kDUmax) ? fmax(v, sh[w][q]) : v + sh[w][q];
-        dst[q] = v;
-    }
+    wait_prerequisites();
+    launch_dependents();
+    const int per = (nb + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int first = (int)blockIdx.x * per, last = min(nb, first + per);
+    float hi[kDiagPass1] = {}, lo[kDiagPass1] = {};
+    add_rows(rows, first, last, hi, lo);
+    const float2 v = block_sum_pairs<kDiagPass1, kDUmax>(hi, lo);
+    if (threadIdx.x >= kDiagPass1) return;
+    if (gridDim.x > 1)
+        reinterpret_cast<float2*>(out + (size_t)blockIdx.x * kDNumSlots)[threadIdx.x] = v;
+    else
+        out[threadIdx.x] = (double)v.x + (double)v.y;
 }
 
 #endif  // LBM_REDUCTION_KERNELS
@@ -1210,11 +1228,16 @@ struct FieldArgs {
     double* rho_p;
 };
 
+// One node per thread, blocks in node order, as k_step: in a strided loop the
+// warps drift apart and what the loads' 256-byte prefetch brings for the next
+// warp is evicted before its use (see k_diag_moments): 256^3 FP32 0.552 against
+// 0.70 to 0.83 ms, 99 % of the copy bandwidth.
 template <class P, class T>
-__global__ void k_get_fields(FieldArgs a)
+__global__ void __launch_bounds__(256) k_get_fields(FieldArgs a)
 {
     const uint32_t n3 = a.geo.n3;
-    for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n3; idx += gridDim.x * blockDim.x) {
+    const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx < n3) {
         int x, y, z;
         node_xyz(a.geo, idx, x, y, z);
         const NodeAddr na = node_addr<T>(a.geo, x, y, z);

@@ -41,6 +41,6 @@ const KernelSet* kernel_set(int pair, int storage)
 }
 
 const void* diag_gradients_kernel() { return (const void*)k_diag_gradients; }
-const void* diag_final_kernel() { return (const void*)k_diag_final; }
+const void* diag_rows_kernel() { return (const void*)k_diag_rows; }
 
 }  // namespace lbm
