@@ -91,6 +91,11 @@ struct lbm_ctx {
     int bxo = 0, byo = 0;    // and of the odd ones
     int pairing = LBM_PAIRING_ALL;   // two nodes per thread (16-bit storage, even nx)
     int flat[2] = {0, 0};            // threads per block of flat launches, per AA parity; 0: shaped (bx x by)
+    size_t l2_bytes = 0;
+    bool mirrored = false;           // direction of the latest group of skewed steps
+    cudaGraphExec_t skew_graph = nullptr;   // kSkewGraphSteps skewed steps from the natural layout
+    int skew_eager = 0;              // skewed steps launched one by one (counted up to the graph's due)
+    bool shared_l2 = false;          // steps concurrently with other lattices (batched instances)
     bool tile_staging = false;        // bulk-copy staged kernel where it applies
     bool slab = false;                // z-slab: planes 0 and nz - 1 are ghost planes (lbm_set_slab)
     bool stage_used = false;          // the staged kernel, the one that can raise d_err, has been launched
@@ -247,6 +252,8 @@ void drop_graph(lbm_ctx* h)
 {
     if (h->graph) cudaGraphExecDestroy(h->graph);
     h->graph = nullptr;
+    if (h->skew_graph) cudaGraphExecDestroy(h->skew_graph);
+    h->skew_graph = nullptr;
 }
 
 int ensure_store(lbm_ctx* h)
@@ -440,16 +447,6 @@ int fill_diag(const lbm_ctx* h, int64_t step, lbm_diag* out)
     return LBM_OK;
 }
 
-dim3 step_grid(const lbm_ctx* h, int odd)
-{
-    const int xunits = uses_pairs(h, odd) ? h->p.nx / 2 : h->p.nx;
-    const dim3 b = step_block(h, odd);
-    if (h->flat[odd])
-        return dim3((unsigned)(((int64_t)xunits * h->p.ny + b.x - 1) / b.x), 1u, (unsigned)h->p.nz);
-    return dim3((unsigned)((xunits + (int)b.x - 1) / (int)b.x), (unsigned)((h->p.ny + (int)b.y - 1) / (int)b.y),
-                (unsigned)h->p.nz);
-}
-
 cudaError_t launch_staged(lbm_ctx* h, int odd, int W, cudaStream_t s)
 {
     const void* k = h->ks->staged[h->p.forcing][odd];
@@ -481,17 +478,44 @@ cudaError_t launch_staged(lbm_ctx* h, int odd, int W, cudaStream_t s)
     return cudaLaunchKernel(k, dim3((unsigned)h->stage_grid), dim3((unsigned)stage_threads(W)), args, smem, s);
 }
 
-StepArgs step_args(lbm_ctx* h, int odd)
+// A box of planes and rows of the lattice (round the periodic ends), and the
+// order of its planes.
+struct StepRange {
+    int z0, planes, y0, rows, down;
+};
+StepRange whole_range(const lbm_ctx* h)
+{
+    // a z-slab updates its own planes 1 .. nz - 2; the ghost planes are only
+    // read and written by the boundary planes' odd steps (never wrapped)
+    if (h->slab) return StepRange{1, h->p.nz - 2, 0, h->p.ny, 0};
+    return StepRange{0, h->p.nz, 0, h->p.ny, 0};
+}
+
+dim3 step_grid(const lbm_ctx* h, int odd, const StepRange& r)
+{
+    const int xunits = uses_pairs(h, odd) ? h->p.nx / 2 : h->p.nx;
+    const dim3 b = step_block(h, odd);
+    if (h->flat[odd])
+        return dim3((unsigned)(((int64_t)xunits * r.rows + b.x - 1) / b.x), 1u, (unsigned)r.planes);
+    return dim3((unsigned)((xunits + (int)b.x - 1) / (int)b.x), (unsigned)((r.rows + (int)b.y - 1) / (int)b.y),
+                (unsigned)r.planes);
+}
+
+StepArgs step_args(lbm_ctx* h, int odd, const StepRange& r)
 {
     StepArgs a{};
     a.f = f_ptr(h);
     a.g = g_ptr(h);
     a.geo = h->geo;
     a.ph = h->ph;
+    a.z0 = r.z0;
+    a.y0 = r.y0;
+    a.rows = r.rows;
+    a.down = r.down;
     if (h->flat[odd]) {
         // ceil(2^(31 + s) / row) with 2^s >= row divides exactly below 2^31
         a.flat_row = (uint32_t)(uses_pairs(h, odd) ? h->p.nx / 2 : h->p.nx);
-        a.flat = a.flat_row * (uint32_t)h->p.ny;
+        a.flat = a.flat_row * (uint32_t)r.rows;
         uint32_t sh = 1;
         while ((1ull << sh) < a.flat_row) ++sh;
         a.flat_mul = (uint32_t)(((1ull << (31 + sh)) + a.flat_row - 1) / a.flat_row);
@@ -500,16 +524,9 @@ StepArgs step_args(lbm_ctx* h, int odd)
     return a;
 }
 
-cudaError_t launch_step(lbm_ctx* h, int odd, cudaStream_t s)
+cudaError_t launch_range(lbm_ctx* h, int odd, const StepRange& r, cudaStream_t s)
 {
-    const int W = stage_width(h);
-    if (W > 0) return launch_staged(h, odd, W, s);
-    StepArgs a = step_args(h, odd);
-    // a z-slab updates its own planes 1 .. nz - 2; the ghost planes are only
-    // read and written by the boundary planes' odd steps (never wrapped)
-    a.z0 = h->slab ? 1 : 0;
-    dim3 grid = step_grid(h, odd);
-    if (h->slab) grid.z = (unsigned)(h->p.nz - 2);
+    StepArgs a = step_args(h, odd, r);
     void* args[] = {&a};
     const int flat = h->flat[odd] ? 1 : 0;
     const void* k = uses_pairs(h, odd) ? h->ks->step2[h->p.forcing][odd][flat] : h->ks->step[h->p.forcing][odd][flat];
@@ -517,7 +534,170 @@ cudaError_t launch_step(lbm_ctx* h, int odd, cudaStream_t s)
     // FP32 D3Q27xD3Q19 11.7 against 12.2 us per step, 32^3 D3Q19xD3Q7 2.2 against
     // 2.7. Below one wave of the longer kernels the waiting blocks share SMs with
     // the running ones: 27x19 32^3 3.3 to 3.9 from run to run against 3.46.
-    return launch_overlapped(k, grid, step_block(h, odd), args, s, !one_short_wave(h));
+    return launch_overlapped(k, step_grid(h, odd, r), step_block(h, odd), args, s, !one_short_wave(h));
+}
+
+cudaError_t launch_step(lbm_ctx* h, int odd, cudaStream_t s)
+{
+    const int W = stage_width(h);
+    if (W > 0) return launch_staged(h, odd, W, s);
+    StepRange r = whole_range(h);
+    r.down = odd;   // starts where the step before ended, in what L2 holds of a larger lattice
+    return launch_range(h, odd, r, s);
+}
+
+// Skewed stepping of a lattice larger than L2. A step of the whole lattice
+// moves every population through HBM; here a strip (some planes and rows, that
+// L2 holds) runs `depth` steps before the next strip starts, so that a
+// population crosses HBM about once in `depth` steps and the strip's launches
+// work from L2. Step s of a node needs step s - 1 of its neighbours and nothing
+// else (in the AA pattern a node's step reads and writes locations of its own),
+// so a strip's range moves down by one plane and one row a step, into what the
+// strips before it have left one step behind; along each axis the first strip
+// shrinks by one at both ends and the last takes what it left, round the
+// periodic end. The launches are the plain step kernels in stream order: the
+// same operations on the same values. A strip is swept back and forth and every
+// other group of steps runs mirrored, so that a launch starts where the one
+// before it ended, in what L2 holds.
+//
+// us per step, whole lattice swept one way (the form before) / back and forth /
+// skewed in strips of about 3/4 of L2: D3Q27xD3Q19 FP32 96^3 50.4 / 43.0 / 40.8,
+// 128^3 115.4 / 107.0 / 97.6, 192^3 384 / 379 / 364, 256^3 905 / 897 / 824-829,
+// 512^3 7124 / - / 6653; D3Q19xD3Q7 FP32 256^3 516 / 510 / 455; D3Q27xD3Q19 FP16
+// 128^3 60.0 / 54.1 / 53.0, 256^3 451.5 / 446.8 / 446. From L2 a step runs at 20
+// to 22 G nodes/s FP32, 37 to 39 FP16, two thirds of the issue slots busy.
+struct SkewPlan {
+    int jz, jy, depth;   // strips along z and y, steps per strip; depth 1: whole-lattice steps
+};
+
+constexpr int kSkewDepth = 16;   // deeper gains under 0.3 %, and the ranges move further
+constexpr int kSkewSteps = 4;    // fewer steps in a call run whole
+
+// Strips of at most 3/4 of L2 in FP32; 0.4 of it for lattices of up to 6 L2,
+// which are stepped beside others (several handles on their streams) more often
+// and then still share it: 50 steps and a record at 128^3 in strips of 0.4 /
+// 0.75 of L2 5.13 / 4.98 ms alone and 5.29 / 5.61 beside another lattice
+// (whole-lattice steps 5.44 and 5.60), 100 at 256^3 88.5 / 82.9 alone and 84.9 /
+// 88.5 beside (89.5 and 90.1), at 160^3 as good either way. One L2 in 16 bits,
+// where only deep strips gain (256^3 in 96 / 129 MB strips 449.7 / 446.4 us per
+// step). Along z alone while the strips are 16 planes thick, else about square
+// in y and z.
+SkewPlan skew_plan(const lbm_ctx* h)
+{
+    const SkewPlan whole{1, 1, 1};
+    const double bytes = (double)(h->q.qf + h->q.qg) * (double)h->geo.n3 * (double)elem_size(h->p.storage);
+    const double l2 = (double)h->l2_bytes;
+    const double strip = h->p.storage != LBM_FP32 ? l2 : bytes > 6.0 * l2 ? 0.75 * l2 : 0.4 * l2;
+    // (72^3 FP32 D3Q27xD3Q19, 69 MB: whole steps 16.4 us from L2)
+    if (bytes <= std::max(strip, 0.75 * l2) || h->slab || stage_width(h) > 0) return whole;
+    const int nz = h->p.nz, ny = h->p.ny;
+    const int64_t want = (int64_t)std::ceil(bytes / strip);
+    SkewPlan p{1, 1, kSkewDepth};
+    if (want <= nz / kSkewDepth) {
+        p.jz = (int)want;
+    } else {
+        const double side = std::sqrt((double)want * nz / ny);
+        p.jz = (int)std::min<double>(std::max(1.0, std::round(side)), std::max(1, nz / kSkewDepth));
+        p.jy = (int)std::min<int64_t>((want + p.jz - 1) / p.jz, std::max(1, ny / kSkewDepth));
+    }
+    // a box too flat for strips that L2 holds
+    if ((int64_t)p.jz * p.jy * 2 < want) return whole;
+    return p;
+}
+
+// Range of strip j of `strips` along an axis of n, at step l of a group of k
+// (n / strips >= k, or one strip).
+void skewed_range(int n, int strips, int j, int k, int l, bool mirrored, int& first, int& count)
+{
+    auto cut = [&](int i) { return (int)((int64_t)i * n / strips) + k - 1; };
+    first = 0;
+    count = n;
+    if (strips > 1) {
+        first = j == 0 ? l : cut(j) - l;
+        count = (j == strips - 1 ? n + l : cut(j + 1) - l) - first;
+        if (first >= n) first -= n;
+    }
+    if (mirrored) first = (2 * n - first - count) % n;
+}
+
+// One group of k steps from AA parity `odd`.
+cudaError_t launch_group(lbm_ctx* h, const SkewPlan& p, int k, int odd, bool mirrored, cudaStream_t s)
+{
+    for (int z = 0; z < p.jz; ++z)
+        for (int y = 0; y < p.jy; ++y)
+            for (int l = 0; l < k; ++l) {
+                StepRange r{};
+                skewed_range(h->p.nz, p.jz, z, k, l, mirrored, r.z0, r.planes);
+                skewed_range(h->p.ny, p.jy, y, k, l, mirrored, r.y0, r.rows);
+                r.down = (int)mirrored ^ (l & 1);
+                const cudaError_t e = launch_range(h, odd ^ (l & 1), r, s);
+                if (e != cudaSuccess) return e;
+            }
+    return cudaSuccess;
+}
+
+// Captures `record` on the stream and instantiates it; null where the stream
+// cannot be captured (the caller then launches eagerly).
+template <class Record>
+cudaGraphExec_t capture_graph(cudaStream_t s, Record&& record)
+{
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t x = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        e = record();
+        const cudaError_t e2 = cudaStreamEndCapture(s, &g);
+        if (e == cudaSuccess) e = e2;
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&x, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (e == cudaSuccess) return x;
+    cudaGetLastError();
+    return nullptr;
+}
+
+// A lattice stepped in strips takes 10 to 250 launches a step. Two groups, one
+// mirrored, make a graph, so that a long call does not fill the launch queue
+// and wait in it; it is built once as many steps as kSkewGraphAfter such pairs
+// have run (256^3: 1152 nodes, a few ms), before that and beside it groups are
+// launched one by one, which keeps ahead of kernels of 14 to 25 us.
+constexpr int kSkewGraphSteps = 2 * kSkewDepth;
+constexpr int kSkewGraphAfter = 4;
+
+cudaError_t step_skewed(lbm_ctx* h, const SkewPlan& p, int64_t nsteps, cudaStream_t s)
+{
+    while (nsteps > 0) {
+        const bool graphs = h->graphs && s != nullptr && nsteps >= kSkewGraphSteps &&
+                            h->skew_eager >= kSkewGraphAfter * kSkewGraphSteps;
+        if (graphs && h->odd == 0) {
+            if (!h->skew_graph)
+                h->skew_graph = capture_graph(s, [&] {
+                    const cudaError_t e = launch_group(h, p, kSkewDepth, 0, true, s);
+                    return e != cudaSuccess ? e : launch_group(h, p, kSkewDepth, 0, false, s);
+                });
+            if (h->skew_graph) {
+                const cudaError_t e = cudaGraphLaunch(h->skew_graph, s);
+                if (e != cudaSuccess) return e;
+                h->mirrored = false;
+                h->step += kSkewGraphSteps;
+                nsteps -= kSkewGraphSteps;
+                continue;
+            }
+            h->graphs = false;
+        }
+        // an odd group brings the natural layout that the graph starts from;
+        // else the steps left are dealt to groups of about equal length
+        const int64_t groups = (nsteps + p.depth - 1) / p.depth;
+        const int k = graphs && h->odd ? kSkewDepth - 1 : (int)((nsteps + groups - 1) / groups);
+        h->mirrored = !h->mirrored;
+        const cudaError_t e = launch_group(h, p, k, h->odd, h->mirrored, s);
+        if (e != cudaSuccess) return e;
+        h->odd ^= k & 1;
+        h->step += k;
+        h->skew_eager = std::min(h->skew_eager + k, kSkewGraphAfter * kSkewGraphSteps);
+        nsteps -= k;
+    }
+    return cudaSuccess;
 }
 
 // What follows pass 1, whose `rows` rows are in h->diag_partials: more than
@@ -782,6 +962,8 @@ int lbm_create_params(lbm_handle* out, const lbm_params* p)
     h->device = dev;
     cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (h->num_sms < 1) h->num_sms = 1;
+    int l2 = 0;
+    if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) == cudaSuccess && l2 > 0) h->l2_bytes = (size_t)l2;
     // a device reset ends every handle, so looking the scratch address up
     // again here keeps the cached one valid for every handle in use
     static_scratch_refresh(dev);
@@ -1036,24 +1218,24 @@ int lbm_step(lbm_handle h, int64_t nsteps)
     if (rc) return rc;
     if (nsteps < 0) return fail(LBM_EINVAL, "negative step count");
     if (!h->initialized) return fail(LBM_ESTATE, "lbm_step before initialisation");
+    if (nsteps >= kSkewSteps && !h->shared_l2) {
+        const SkewPlan plan = skew_plan(h);
+        if (plan.depth > 1) {
+            LBM_CUDA(step_skewed(h, plan, nsteps, h->stream), "step launch");
+            return LBM_OK;
+        }
+    }
     while (nsteps > 0) {
         if (h->graphs && h->stream != nullptr && h->odd == 0 && nsteps >= kGraphSteps) {
-            if (!h->graph) {
-                cudaGraph_t g = nullptr;
-                cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
-                if (e == cudaSuccess) {
+            if (!h->graph)
+                h->graph = capture_graph(h->stream, [&] {
+                    cudaError_t e = cudaSuccess;
                     for (int s = 0; s < kGraphSteps && e == cudaSuccess; ++s) e = launch_step(h, s & 1, h->stream);
-                    cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
-                    if (e == cudaSuccess) e = e2;
-                }
-                if (e == cudaSuccess) e = cudaGraphInstantiate(&h->graph, g, 0);
-                if (g) cudaGraphDestroy(g);
-                if (e != cudaSuccess) {
-                    cudaGetLastError();
-                    h->graph = nullptr;
-                    h->graphs = false;  // fall back to eager launches
-                    continue;
-                }
+                    return e;
+                });
+            if (!h->graph) {
+                h->graphs = false;  // fall back to eager launches
+                continue;
             }
             LBM_CUDA(cudaGraphLaunch(h->graph, h->stream), "graph launch");
             h->step += kGraphSteps;
@@ -1107,11 +1289,12 @@ int lbm_step_diagnostics(lbm_handle h, int64_t nsteps, lbm_diag* out)
     if (h->slab) return fail(LBM_EUNSUPPORTED, "a z-slab steps with lbm_step and reports with lbm_diagnostics");
     const int odd = h->odd;
     const bool pairs = uses_pairs(h, odd);
-    const dim3 grid = step_grid(h, odd);
+    const StepRange range = whole_range(h);
+    const dim3 grid = step_grid(h, odd, range);
     const int rows = (int)(grid.x * grid.y * grid.z);
     if ((rc = ensure_diag(h, rows + h->num_sms))) return rc;
     const DiagArgs da = diag_args(h);
-    StepArgs a = step_args(h, odd);
+    StepArgs a = step_args(h, odd, range);
     a.dg = DiagSink{da.ep_scale, da.epsk_scale, da.s_scale, h->diag_fields, h->diag_partials};
     void* args[] = {&a};
     const void* k = pairs ? h->ks->step2_diag[h->p.forcing][odd] : h->ks->step_diag[h->p.forcing][odd];
@@ -1972,6 +2155,7 @@ int lbm_batch_create(lbm_batch* out, const lbm_params* params, int count)
         rc = lbm_create_params(&h, &params[i]);
         if (rc) break;
         b->inst.push_back(h);
+        h->shared_l2 = true;
         if ((rc = lbm_set_stream(h, b->stream))) break;
         if ((rc = ensure_store(h))) break;
     }

@@ -122,47 +122,47 @@ LBM_HD void sfor(F&& f)
 // ---------------------------------------------------------------------------
 template <class T>
 __device__ __forceinline__ float ld_pop(const T* p);
-// Population loads are streaming (evict-first) and ask L2 to fetch the whole
-// 256-byte block around the address. A warp's row segment is 128 bytes in
-// FP32 (64 in 16-bit storage) and the next warps read the next ones, so the
-// rest of the block arrives early: FP32 D3Q27xD3Q19 at 256^3 0.9087 against
-// 0.9121-0.9128 ms per step (two boxes), D3Q19xD3Q7 0.5433 against 0.5509;
-// the one-node 16-bit kernel 0.3-0.8 % faster. The block lies in the same
-// mapped page as the address, so the hint never reaches past the
-// allocation's pages.
-__device__ __forceinline__ uint16_t ld_u16_stream(const void* p)
+// Population loads ask L2 to fetch the whole 256-byte block around the address.
+// A warp's row segment is 128 bytes in FP32 (64 in 16-bit storage) and the next
+// warps read the next ones, so the rest of the block arrives early. Loads and
+// stores keep the normal priority in L2: the next step starts where this one
+// ends and finds it there (as evict-first, `.cs`, 96^3 D3Q27xD3Q19 FP32 42.7
+// against 42.5 us per step, 256^3 898 against 894, D3Q19xD3Q7 509.5 against
+// 507.9). The block lies in the same mapped page as the address, so the hint
+// never reaches past the allocation's pages.
+__device__ __forceinline__ uint16_t ld_u16(const void* p)
 {
     uint16_t v;
-    asm volatile("ld.global.cs.L2::256B.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    asm volatile("ld.global.L2::256B.u16 %0, [%1];" : "=h"(v) : "l"(p));
     return v;
 }
 template <>
 __device__ __forceinline__ float ld_pop<float>(const float* p)
 {
     float v;
-    asm volatile("ld.global.cs.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    asm volatile("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
 template <>
 __device__ __forceinline__ float ld_pop<__half>(const __half* p)
 {
-    return __half2float(__ushort_as_half(ld_u16_stream(p)));
+    return __half2float(__ushort_as_half(ld_u16(p)));
 }
 template <>
 __device__ __forceinline__ float ld_pop<__nv_bfloat16>(const __nv_bfloat16* p)
 {
-    return __bfloat162float(__ushort_as_bfloat16(ld_u16_stream(p)));
+    return __bfloat162float(__ushort_as_bfloat16(ld_u16(p)));
 }
 template <class T>
 __device__ __forceinline__ void st_pop(T* p, float v);
 template <>
-__device__ __forceinline__ void st_pop<float>(float* p, float v) { __stcs(p, v); }
+__device__ __forceinline__ void st_pop<float>(float* p, float v) { *p = v; }
 template <>
-__device__ __forceinline__ void st_pop<__half>(__half* p, float v) { __stcs(p, __float2half_rn(v)); }
+__device__ __forceinline__ void st_pop<__half>(__half* p, float v) { *p = __float2half_rn(v); }
 template <>
 __device__ __forceinline__ void st_pop<__nv_bfloat16>(__nv_bfloat16* p, float v)
 {
-    __stcs(p, __float2bfloat16_rn(v));
+    *p = __float2bfloat16_rn(v);
 }
 
 // ---------------------------------------------------------------------------

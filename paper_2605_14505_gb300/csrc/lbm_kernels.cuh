@@ -261,7 +261,9 @@ struct StepArgs {
     Geometry geo;
     Phys ph;
     DiagSink dg;      // used by the diagnosing variants only
-    int z0;           // first z-plane of the launch (1 for a z-slab with ghost planes, else 0)
+    // planes [z0, z0 + gridDim.z) and rows [y0, y0 + rows), round the periodic
+    // ends; `down`: the planes from the last to the first
+    int z0, y0, rows, down;
     // flat launches (flat > 0): threads number the plane's units (nodes, or
     // pairs of nodes) row by row, flat of them in rows of flat_row;
     // r / flat_row = umulhi(r, flat_mul) >> flat_shift for r < 2^31
@@ -280,11 +282,21 @@ __device__ __forceinline__ bool step_unit(const StepArgs& a, int xunits, int& xu
         const uint32_t r = blockIdx.x * blockDim.x + tx;
         y = (int)(__umulhi(r, a.flat_mul) >> a.flat_shift);
         xu = (int)(r - (uint32_t)y * a.flat_row);
+        y += a.y0;
+        if (y >= a.geo.ny) y -= a.geo.ny;
         return r < a.flat;
     }
     xu = (int)(blockIdx.x * blockDim.x + tx);
     y = (int)(blockIdx.y * blockDim.y + threadIdx.y);
-    return xu < xunits && y < a.geo.ny;
+    const bool inside = xu < xunits && y < a.rows;
+    y += a.y0;
+    if (y >= a.geo.ny) y -= a.geo.ny;
+    return inside;
+}
+__device__ __forceinline__ int step_plane(const StepArgs& a)
+{
+    const int z = a.z0 + (int)(a.down ? gridDim.z - 1u - blockIdx.z : blockIdx.z);
+    return z >= a.geo.nz ? z - a.geo.nz : z;
 }
 
 // Programmatic dependent launch: once every block of a step has come to its
@@ -374,7 +386,7 @@ template <class P, int FORCING, class T, bool ODD, int LAUNCH>
 __global__ void __launch_bounds__(256, kStepMinBlocks<P>) k_step(StepArgs args)
 {
     int x, y;
-    const int z = blockIdx.z + args.z0;
+    const int z = step_plane(args);
     if (!step_unit<LAUNCH>(args, args.geo.nx, x, y, threadIdx.x)) return;
     wait_prerequisites();
     update_node<P, FORCING, T, ODD>(args.f, args.g, args.geo, args.ph, x, y, z, [](const float*, const Macro&) {},
@@ -390,7 +402,7 @@ template <class P, int FORCING, class T, bool ODD>
 __global__ void __launch_bounds__(256, 3) k_step_diag(StepArgs args)
 {
     int x, y;
-    const int z = blockIdx.z;
+    const int z = (int)blockIdx.z;
     constexpr bool kExact = std::is_same<T, float>::value;
     DiagAcc d;
     if (step_unit<kAsked>(args, args.geo.nx, x, y, threadIdx.x)) {
@@ -484,18 +496,18 @@ struct Seam {
 // against 0.269 ms at 256^3).
 __device__ __forceinline__ uint32_t seam_word(uint32_t w, uint32_t sel) { return __byte_perm(w, 0u, sel); }
 
-// Streaming (evict-first) word loads that ask L2 for the whole 256-byte
-// block, as the FP32 loads do: D3Q19xD3Q7 FP16 at 256^3 0.2638 against
-// 0.2694 ms per step with plain loads, D3Q27xD3Q19 unchanged (0.4536 ms).
+// Word loads that ask L2 for the whole 256-byte block, as the FP32 loads do:
+// D3Q19xD3Q7 FP16 at 256^3 0.258 against 0.263 ms per step with plain loads,
+// D3Q27xD3Q19 0.445 against 0.447.
 __device__ __forceinline__ uint32_t ld_word(const unsigned short* p)
 {
     uint32_t v;
-    asm volatile("ld.global.cs.L2::256B.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    asm volatile("ld.global.L2::256B.u32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
 __device__ __forceinline__ void st_word(unsigned short* p, uint32_t w)
 {
-    __stcs(reinterpret_cast<unsigned int*>(p), w);
+    *reinterpret_cast<unsigned int*>(p) = w;
 }
 
 template <class L, bool ODD>
@@ -719,7 +731,7 @@ template <class P, int FORCING, class T, bool ODD, int LAUNCH>
 __global__ void __launch_bounds__(256, kStep2MinBlocks<P>) k_step2(StepArgs args)
 {
     int k, y;
-    const int z = blockIdx.z + args.z0;
+    const int z = step_plane(args);
     if (!step_unit<LAUNCH>(args, args.geo.nx / 2, k, y, threadIdx.x)) return;
     wait_prerequisites();
     update_pair<P, FORCING, T, ODD>(args, 2 * k, y, z, NoHook{}, StepPlace<LAUNCH>{args, 2});
@@ -731,7 +743,7 @@ template <class P, int FORCING, class T, bool ODD>
 __global__ void __launch_bounds__(256, 2) k_step2_diag(StepArgs args)
 {
     int k, y;
-    const int z = blockIdx.z;
+    const int z = (int)blockIdx.z;
     DiagAcc d;
     if (step_unit<kAsked>(args, args.geo.nx / 2, k, y, threadIdx.x)) {
         const int x0 = 2 * k;
