@@ -69,6 +69,10 @@ constexpr int kGraphSteps = 64;   // even number: the graph starts and ends in n
 // scratch on `device`, which must be current; defined with the array below.
 void static_scratch_refresh(int device);
 
+// What a lattice may take of L2: as it comes; steps beside others of its batch,
+// whole lattices only; has the GPU to itself in its batch.
+enum class L2Use { unknown, shared, alone };
+
 }  // namespace
 
 struct lbm_ctx {
@@ -95,7 +99,7 @@ struct lbm_ctx {
     bool mirrored = false;           // direction of the latest group of skewed steps
     cudaGraphExec_t skew_graph = nullptr;   // kSkewGraphSteps skewed steps from the natural layout
     int skew_eager = 0;              // skewed steps launched one by one (counted up to the graph's due)
-    bool shared_l2 = false;          // steps concurrently with other lattices (batched instances)
+    L2Use l2 = L2Use::unknown;
     bool tile_staging = false;        // bulk-copy staged kernel where it applies
     bool slab = false;                // z-slab: planes 0 and nz - 1 are ghost planes (lbm_set_slab)
     bool stage_used = false;          // the staged kernel, the one that can raise d_err, has been launched
@@ -587,7 +591,7 @@ SkewPlan skew_plan(const lbm_ctx* h)
     const SkewPlan whole{1, 1, 1};
     const double bytes = (double)(h->q.qf + h->q.qg) * (double)h->geo.n3 * (double)elem_size(h->p.storage);
     const double l2 = (double)h->l2_bytes;
-    const double strip = h->p.storage != LBM_FP32 ? l2 : bytes > 6.0 * l2 ? 0.75 * l2 : 0.4 * l2;
+    const double strip = h->p.storage != LBM_FP32 ? l2 : bytes > 6.0 * l2 || h->l2 == L2Use::alone ? 0.75 * l2 : 0.4 * l2;
     // (72^3 FP32 D3Q27xD3Q19, 69 MB: whole steps 16.4 us from L2)
     if (bytes <= std::max(strip, 0.75 * l2) || h->slab || stage_width(h) > 0) return whole;
     const int nz = h->p.nz, ny = h->p.ny;
@@ -1218,7 +1222,7 @@ int lbm_step(lbm_handle h, int64_t nsteps)
     if (rc) return rc;
     if (nsteps < 0) return fail(LBM_EINVAL, "negative step count");
     if (!h->initialized) return fail(LBM_ESTATE, "lbm_step before initialisation");
-    if (nsteps >= kSkewSteps && !h->shared_l2) {
+    if (nsteps >= kSkewSteps && h->l2 != L2Use::shared) {
         const SkewPlan plan = skew_plan(h);
         if (plan.depth > 1) {
             LBM_CUDA(step_skewed(h, plan, nsteps, h->stream), "step launch");
@@ -1832,6 +1836,9 @@ struct lbm_batch_ctx {
     // with its own single-lattice step kernel; streams and join events are
     // created on first use
     std::vector<std::vector<int>> chain_of;
+    // the same driver's rounds: instances that L2 holds together run all steps
+    // of a call before the next round's
+    std::vector<std::vector<int>> rounds;
     std::vector<cudaStream_t> cstream;
     std::vector<cudaEvent_t> cjoin;
     int bx = 32, by = 8;
@@ -2024,24 +2031,80 @@ cudaError_t batch_ensure_chains(lbm_batch_ctx* b)
     return cudaSuccess;
 }
 
-// Per-instance driver: nsteps steps of every instance, each by lbm_step on
-// its chain's stream (the instance's own 64-step graph replays, eager steps
-// outside them), the chains forked from and joined back to b->stream.
-int batch_step_instances(lbm_batch_ctx* b, int64_t nsteps)
+// Rounds of the per-instance driver: instances in order of size, as many to a
+// round as 3/4 of L2 holds, at least one. All 64 lattices of a size, pair,
+// forcing and Froude number sweep (32^3 to 96^3, 2.6 GB) at once leave nothing
+// in L2 from step to step (885 us a step of all of them, 98 % of the copy
+// bandwidth); in rounds all but the 96^3 D3Q27xD3Q19 ones step from L2, and
+// those, one to a round, in skewed strips: 728 us.
+void batch_build_rounds(lbm_batch_ctx* b)
 {
-    LBM_CUDA(batch_ensure_chains(b), "batch chain streams");
+    if (!b->rounds.empty()) return;
+    std::vector<int> order(b->inst.size());
+    for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int a, int c) { return b->inst[a]->store_bytes > b->inst[c]->store_bytes; });
+    const size_t budget = b->inst[0]->l2_bytes / 4 * 3;
+    size_t held = 0;
+    for (int i : order) {
+        const size_t bytes = b->inst[i]->store_bytes;
+        if (b->rounds.empty() || held + bytes > budget) {
+            b->rounds.emplace_back();
+            held = 0;
+        }
+        b->rounds.back().push_back(i);
+        held += bytes;
+    }
+}
+
+// work(h) for the instances of each chain with h on the chain's stream, the
+// chains forked from and joined back to b->stream.
+template <class Work>
+int batch_run_chains(lbm_batch_ctx* b, const std::vector<std::vector<int>>& chains, Work&& work)
+{
     LBM_CUDA(cudaEventRecord(b->vfork, b->stream), "batch fork");
-    for (size_t c = 0; c < b->chain_of.size(); ++c) {
+    for (size_t c = 0; c < chains.size(); ++c) {
         LBM_CUDA(cudaStreamWaitEvent(b->cstream[c], b->vfork, 0), "batch fork wait");
-        for (int i : b->chain_of[c]) {
+        for (int i : chains[c]) {
             lbm_ctx* h = b->inst[i];
             h->stream = b->cstream[c];
-            const int rc = lbm_step(h, nsteps);
+            const int rc = work(h);
             h->stream = b->stream;
             if (rc) return rc;
         }
         LBM_CUDA(cudaEventRecord(b->cjoin[c], b->cstream[c]), "batch join");
         LBM_CUDA(cudaStreamWaitEvent(b->stream, b->cjoin[c], 0), "batch join wait");
+    }
+    return LBM_OK;
+}
+
+// Instances dealt to at most `most` chains.
+std::vector<std::vector<int>> deal_chains(const std::vector<int>& instances, size_t most)
+{
+    std::vector<std::vector<int>> chains(std::min(instances.size(), most));
+    for (size_t k = 0; k < instances.size(); ++k) chains[k % chains.size()].push_back(instances[k]);
+    return chains;
+}
+
+// A call of one step keeps nothing in L2 and runs all instances at once (the
+// sweep above in calls of 1 / 2 / 4 / 100 steps: 970 / 956 / 821 / 728 us a step;
+// 4 steps all at once 1007).
+constexpr int64_t kRoundSteps = 2;
+
+int batch_step_instances(lbm_batch_ctx* b, int64_t nsteps)
+{
+    LBM_CUDA(batch_ensure_chains(b), "batch chain streams");
+    // lbm_step on the chain's stream: the instance's own graph replays, eager steps outside them
+    if (nsteps < kRoundSteps) return batch_run_chains(b, b->chain_of, [&](lbm_ctx* h) { return lbm_step(h, nsteps); });
+    batch_build_rounds(b);
+    for (const std::vector<int>& round : b->rounds) {
+        const int rc = batch_run_chains(b, deal_chains(round, b->chain_of.size()), [&](lbm_ctx* h) {
+            if (round.size() == 1) h->l2 = L2Use::alone;
+            const int r = lbm_step(h, nsteps);
+            h->l2 = L2Use::shared;
+            return r;
+        });
+        if (rc) return rc;
     }
     return LBM_OK;
 }
@@ -2155,7 +2218,7 @@ int lbm_batch_create(lbm_batch* out, const lbm_params* params, int count)
         rc = lbm_create_params(&h, &params[i]);
         if (rc) break;
         b->inst.push_back(h);
-        h->shared_l2 = true;
+        h->l2 = L2Use::shared;
         if ((rc = lbm_set_stream(h, b->stream))) break;
         if ((rc = ensure_store(h))) break;
     }
@@ -2339,9 +2402,19 @@ int lbm_batch_diagnostics(lbm_batch b, lbm_diag* out)
     for (lbm_ctx* h : b->inst) {
         if (!h->initialized) return fail(LBM_ESTATE, "diagnostics before initialisation");
     }
-    // every instance's kernels first, then one wait (one each: 64 instances 3.3 ms)
-    for (lbm_ctx* h : b->inst)
-        if ((rc = enqueue_diagnostics(h))) return rc;
+    // every instance's kernels first, on several streams, then one wait (one
+    // instance after the other with a wait each: 64 instances 3.3 ms)
+    if (b->stream != nullptr) {
+        LBM_CUDA(batch_ensure_chains(b), "batch chain streams");
+        batch_build_rounds(b);
+        std::vector<int> order;
+        for (const std::vector<int>& round : b->rounds) order.insert(order.end(), round.begin(), round.end());
+        rc = batch_run_chains(b, deal_chains(order, std::min<size_t>(b->cstream.size(), 8)), enqueue_diagnostics);
+        if (rc) return rc;
+    } else {
+        for (lbm_ctx* h : b->inst)
+            if ((rc = enqueue_diagnostics(h))) return rc;
+    }
     int worst = LBM_OK;
     for (size_t i = 0; i < b->inst.size(); ++i) {
         LBM_CUDA(cudaStreamSynchronize(b->inst[i]->stream), "diagnostics");
