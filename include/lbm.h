@@ -221,7 +221,10 @@ int lbm_prefetch_fields(lbm_handle h, const double* rho, const double* u, const 
 int lbm_init_prefetched(lbm_handle h);
 
 /* Advance nsteps >= 0 time steps (Eqs. 5, 11: collide, then stream) with
- * the in-place AA pattern; asynchronous on the handle's stream. */
+ * the in-place AA pattern; asynchronous on the handle's stream. A lattice
+ * larger than L2 is stepped in strips that L2 holds, several steps each
+ * (calls of at least 4 steps); the populations are those of whole-lattice
+ * steps, bit for bit. */
 int lbm_step(lbm_handle h, int64_t nsteps);
 
 /* Block until the handle's stream (and its prefetch copies) are idle;
@@ -334,7 +337,10 @@ int lbm_storage_rule(const lbm_diag* ref, const lbm_diag* cand, int64_t count, i
  * thread along x covers two nodes. Each AA parity has its own shape:
  * lbm_set_block sets both, lbm_get_block returns the even steps' shape (the
  * default odd-step shape of the D3Q27xD3Q19 two-nodes-per-thread kernel is
- * one row of 128 threads, its even-step shape 64 x 2). */
+ * one row of 128 threads, its even-step shape 64 x 2). Where it leaves
+ * fewer threads idle (row lengths that fill no shape) the default is a flat
+ * launch, rows numbered through, whatever lbm_get_block returns;
+ * lbm_set_block ends it, lbm_autotune times it beside the shapes. */
 int lbm_set_block(lbm_handle h, int bx, int by);
 int lbm_get_block(lbm_handle h, int* bx, int* by);
 
@@ -434,7 +440,7 @@ int lbm_set_slab(lbm_handle h, int enable);
 int lbm_halo_bytes(lbm_handle h, size_t* bytes);
 
 /* Device buffers (lbm_halo_bytes each, on the handle's device). Enqueued on
- * the handle's stream (device-to-device copies, one per slot and plane);
+ * the handle's stream (one kernel for both buffers, of any alignment);
  * return without waiting. LBM_ESTATE without slab mode or store; LBM_EINVAL
  * for another phase, or a buffer that is null or not device memory of the
  * handle's device. */
@@ -458,11 +464,10 @@ int lbm_destroy(lbm_handle h);
  *    finished step s - 1 (a per-instance completion count), so instances never
  *    wait for each other and there is no grid-wide barrier. Every wait is
  *    bounded. The launch is replayed from a CUDA graph;
- *  - per instance: each instance advanced by its own single-lattice step
- *    kernel (its own launch shape), replayed from a CUDA graph of 64 steps in
- *    which every instance's chain of steps is its own branch (up to 128
- *    branches, largest instances first; instances share no memory, so the
- *    branches overlap and fill each other's tails);
+ *  - per instance: each instance advanced by lbm_step (its own launch shape
+ *    and graphs) on one of up to 128 streams. A call of several steps runs in
+ *    rounds of as many instances as L2 holds, largest first, all steps of the
+ *    call per round; instances share no memory, so those of a round overlap;
  *  - per step: one launch per (pair, forcing) variant over that variant's
  *    tiles, replayed the same way with one branch per variant.
  * Instances may differ in size, pair (D3Q27xD3Q19, D3Q19xD3Q7), forcing and
@@ -494,7 +499,7 @@ int lbm_batch_set_stream(lbm_batch b, void* stream);
  * launch's parameter block: LBM_EUNSUPPORTED beyond, and such batches start
  * in LBM_BATCH_PER_STEP), LBM_BATCH_PER_STEP (one launch per variant and
  * step, replayed from a CUDA graph of 64 steps) or LBM_BATCH_INSTANCES (each
- * instance's own step kernel, one graph branch per instance). */
+ * instance's own steps, in rounds of instances that L2 holds). */
 int lbm_batch_set_mode(lbm_batch b, int mode, int steps_per_launch);
 
 /* Tile shape of the per-step driver: bx in {16, 32, 64, 128} nodes along x,

@@ -211,6 +211,7 @@ void pick_block(const lbm_ctx* h, int odd, int& bx, int& by)
     while (bx * 2 <= want && bx * 2 <= xunits) bx *= 2;
     by = threads / bx;
     while (by > 1 && by / 2 >= h->p.ny) by /= 2;
+    while (bx * by < 256 && (h->p.ny + by - 1) / by > 65535) by *= 2;   // rows of blocks within the grid's limit
 }
 
 // Threads per block of a flat launch (the plane's units numbered through, row
