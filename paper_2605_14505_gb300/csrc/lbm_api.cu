@@ -594,7 +594,7 @@ SkewPlan skew_plan(const lbm_ctx* h)
     const double l2 = (double)h->l2_bytes;
     const double strip = h->p.storage != LBM_FP32 ? l2 : bytes > 6.0 * l2 || h->l2 == L2Use::alone ? 0.75 * l2 : 0.4 * l2;
     // (72^3 FP32 D3Q27xD3Q19, 69 MB: whole steps 16.4 us from L2)
-    if (bytes <= std::max(strip, 0.75 * l2) || h->slab || stage_width(h) > 0) return whole;
+    if (strip <= 0.0 || bytes <= std::max(strip, 0.75 * l2) || h->slab || stage_width(h) > 0) return whole;
     const int nz = h->p.nz, ny = h->p.ny;
     const int64_t want = (int64_t)std::ceil(bytes / strip);
     SkewPlan p{1, 1, kSkewDepth};
@@ -2049,7 +2049,7 @@ void batch_build_rounds(lbm_batch_ctx* b)
     size_t held = 0;
     for (int i : order) {
         const size_t bytes = b->inst[i]->store_bytes;
-        if (b->rounds.empty() || held + bytes > budget) {
+        if (b->rounds.empty() || (budget > 0 && held + bytes > budget)) {
             b->rounds.emplace_back();
             held = 0;
         }
