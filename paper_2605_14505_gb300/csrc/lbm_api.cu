@@ -488,6 +488,10 @@ cudaError_t launch_staged(lbm_ctx* h, int odd, int W, cudaStream_t s)
 struct StepRange {
     int z0, planes, y0, rows, down;
 };
+size_t store_need(const lbm_ctx* h)
+{
+    return (size_t)(h->q.qf + h->q.qg) * h->geo.n3 * elem_size(h->p.storage);
+}
 StepRange whole_range(const lbm_ctx* h)
 {
     // a z-slab updates its own planes 1 .. nz - 2; the ghost planes are only
@@ -547,7 +551,10 @@ cudaError_t launch_step(lbm_ctx* h, int odd, cudaStream_t s)
     const int W = stage_width(h);
     if (W > 0) return launch_staged(h, odd, W, s);
     StepRange r = whole_range(h);
-    r.down = odd;   // starts where the step before ended, in what L2 holds of a larger lattice
+    // of a lattice that L2 does not hold well a step starts where the one before
+    // ended, in what is there; a smaller one keeps its blocks on their SMs (32^3
+    // FP32 D3Q27xD3Q19 3.5 us per step against 3.5 to 3.7 alternating)
+    r.down = odd && 2 * store_need(h) > h->l2_bytes;
     return launch_range(h, odd, r, s);
 }
 
@@ -590,11 +597,15 @@ constexpr int kSkewSteps = 4;    // fewer steps in a call run whole
 SkewPlan skew_plan(const lbm_ctx* h)
 {
     const SkewPlan whole{1, 1, 1};
-    const double bytes = (double)(h->q.qf + h->q.qg) * (double)h->geo.n3 * (double)elem_size(h->p.storage);
+    const double bytes = (double)store_need(h);
     const double l2 = (double)h->l2_bytes;
     const double strip = h->p.storage != LBM_FP32 ? l2 : bytes > 6.0 * l2 || h->l2 == L2Use::alone ? 0.75 * l2 : 0.4 * l2;
     // (72^3 FP32 D3Q27xD3Q19, 69 MB: whole steps 16.4 us from L2)
     if (strip <= 0.0 || bytes <= std::max(strip, 0.75 * l2) || h->slab || stage_width(h) > 0) return whole;
+    // 16 bits with one node per thread (odd nx) are bound by issue: strips' last
+    // waves cost more than HBM traffic saves (27x19 FP16 171^3 167 against 176 us
+    // whole, 225^3 480 against 470, 401^3 2740 against 2641)
+    if (h->p.storage != LBM_FP32 && !uses_pairs(h, 0) && bytes > 6.0 * l2) return whole;
     const int nz = h->p.nz, ny = h->p.ny;
     const int64_t want = (int64_t)std::ceil(bytes / strip);
     SkewPlan p{1, 1, kSkewDepth};
