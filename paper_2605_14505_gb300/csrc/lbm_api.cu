@@ -195,17 +195,23 @@ bool one_short_wave(const lbm_ctx* h) { return h->q.qf + h->q.qg >= 38 && step_w
 // ms, D3Q19xD3Q19 0.751 / 0.768 ms, against 0.520 / 0.528 and 0.758 / 0.776
 // as 128 on both), and for D3Q27xD3Q27 (two 128-register blocks per SM) one
 // row of 64 on even steps and 128 on odd steps (1.058 / 1.096 ms against
-// 1.072 / 1.155 ms as 256).
+// 1.072 / 1.155 ms as 256). Below 20 waves 128 threads: the last, partly filled
+// wave then weighs less than the row order gains (27x19 / 19x7 FP32 at 64^3 11.9
+// / 7.5 us against 12.9 / 7.7 with 256, at 128^3 117.3 / 67.1 against 118.4 /
+// 67.3), and below one wave of the longer kernels 64 (27x19 Guo 32^3, 200 steps
+// and a record: 760 us; 128 757; 256 728 to 769 with where its few blocks land).
 void pick_block(const lbm_ctx* h, int odd, int& bx, int& by)
 {
     const bool pairs = uses_pairs(h, odd);
     const int xunits = pairs ? h->p.nx / 2 : h->p.nx;
     const int qsum = h->q.qf + h->q.qg;
     const bool big = qsum >= 46;
-    const int threads = pairs || (qsum <= 46 && step_waves(h) < 20.0 && !one_short_wave(h)) ? 128
-                        : qsum > 46                                                     ? (odd ? 128 : 64)
-                        : (odd && qsum <= 34)                                           ? 128
-                                                                                        : 256;
+    const int threads = pairs                                ? 128
+                        : qsum <= 46 && one_short_wave(h)    ? 64
+                        : qsum <= 46 && step_waves(h) < 20.0 ? 128
+                        : qsum > 46                          ? (odd ? 128 : 64)
+                        : (odd && qsum <= 34)                ? 128
+                                                             : 256;
     const int want = pairs ? ((odd && big) ? 128 : 64) : threads;
     bx = 32;
     while (bx * 2 <= want && bx * 2 <= xunits) bx *= 2;
@@ -552,8 +558,8 @@ cudaError_t launch_step(lbm_ctx* h, int odd, cudaStream_t s)
     if (W > 0) return launch_staged(h, odd, W, s);
     StepRange r = whole_range(h);
     // of a lattice that L2 does not hold well a step starts where the one before
-    // ended, in what is there; a smaller one keeps its blocks on their SMs (32^3
-    // FP32 D3Q27xD3Q19 3.5 us per step against 3.5 to 3.7 alternating)
+    // ended, in what is there; a smaller one keeps its blocks on their SMs (27x19
+    // Guo 32^3, 200 steps and a record: 760 us, alternating 778)
     r.down = odd && 2 * store_need(h) > h->l2_bytes;
     return launch_range(h, odd, r, s);
 }
