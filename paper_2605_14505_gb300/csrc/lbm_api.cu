@@ -346,19 +346,29 @@ dim3 gradient_grid(const lbm_ctx* h, int& planes)
 // `rows` rows), pass-2 rows, the totals in pinned memory and their event.
 int ensure_diag(lbm_ctx* h, int rows)
 {
-    if (!h->diag_fields) {
-        size_t fbytes = 4 * (size_t)h->geo.n3 * sizeof(float);
+    if (!h->diag_event) {   // the handle gets all of it or, where a part fails, nothing
         int planes = 0;
         const dim3 g = gradient_grid(h, planes);
         const size_t pairs = (size_t)g.x * g.y * kDiagPass2;
-        if (cudaMalloc(&h->diag_fields, fbytes) != cudaSuccess ||
-            cudaMalloc(&h->diag_grad, (pairs + 1) * sizeof(float2)) != cudaSuccess ||
-            cudaMemsetAsync(h->diag_grad + pairs, 0, sizeof(float2), h->stream) != cudaSuccess ||
-            cudaMallocHost(&h->diag_host, 16 * sizeof(double)) != cudaSuccess ||
-            cudaEventCreateWithFlags(&h->diag_event, cudaEventDisableTiming) != cudaSuccess) {
+        float* fields = nullptr;
+        float2* grad = nullptr;
+        double* host = nullptr;
+        cudaEvent_t event = nullptr;
+        if (cudaMalloc(&fields, 4 * (size_t)h->geo.n3 * sizeof(float)) != cudaSuccess ||
+            cudaMalloc(&grad, (pairs + 1) * sizeof(float2)) != cudaSuccess ||
+            cudaMemsetAsync(grad + pairs, 0, sizeof(float2), h->stream) != cudaSuccess ||
+            cudaMallocHost(&host, 16 * sizeof(double)) != cudaSuccess ||
+            cudaEventCreateWithFlags(&event, cudaEventDisableTiming) != cudaSuccess) {
             cudaGetLastError();
+            if (fields) cudaFree(fields);
+            if (grad) cudaFree(grad);
+            if (host) cudaFreeHost(host);
             return fail(LBM_ENOMEM, "diagnostics scratch allocation failed");
         }
+        h->diag_fields = fields;
+        h->diag_grad = grad;
+        h->diag_host = host;
+        h->diag_event = event;
     }
     if (h->diag_rows < rows) {
         if (h->diag_partials) {

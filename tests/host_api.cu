@@ -1,0 +1,85 @@
+// Checks of the library's host code on the CPU: every object of liblbm.so linked
+// with tests/host_runtime.cpp in place of the CUDA runtime.
+//
+//   host_api <check> [arguments]     prints its findings; see tests/test_host_api.py
+#include <cstdio>
+#include <cstdlib>
+#include <string>
+#include <vector>
+
+#include "host_runtime.h"
+#include "lbm.h"
+#include "lbm_kernels.cuh"
+
+namespace {
+
+lbm_handle make(int nx, int ny, int nz, int pair, int storage, int forcing = LBM_SHAN_CHEN)
+{
+    lbm_params p;
+    lbm_params_from_physics(&p, nx, ny, nz, pair, forcing, 100.0, 1.0, 1.0, 0.04);
+    p.storage = storage;
+    lbm_handle h = nullptr;
+    if (lbm_create_params(&h, &p)) std::printf("create: %s\n", lbm_last_error());
+    return h;
+}
+
+void start(lbm_handle h)
+{
+    lbm_params p;
+    lbm_get_params(h, &p);
+    std::vector<double> ones(3 * (size_t)p.nx * p.ny * p.nz, 1.0);
+    if (lbm_init_fields(h, ones.data(), ones.data(), ones.data(), nullptr, nullptr, 0.0))
+        std::printf("init: %s\n", lbm_last_error());
+}
+
+// A record after a failed one: the k-th allocation of the first call fails, the
+// second call has everything in place. One line per k until no call fails.
+int record_scratch(int fused)
+{
+    for (int k = 0;; ++k) {
+        lbm_handle h = make(16, 16, 16, LBM_D3Q19_D3Q7, LBM_FP32);
+        start(h);
+        lbm_diag d;
+        auto record = [&] { return fused ? lbm_step_diagnostics(h, 1, &d) : lbm_diagnostics(h, &d); };
+        g_work.clear();
+        g_fail_in = k;
+        const int first = record();
+        const bool failed = g_fail_in < 0;
+        g_fail_in = -1;
+        size_t launches = 0;
+        for (const Work& w : g_work) launches += w.kind == Work::kLaunch;
+        const int second = record();
+        bool scratch = true;
+        std::set<void*> cleared;
+        for (size_t i = 0; i < g_work.size(); ++i) {
+            const Work& w = g_work[i];
+            if (w.kind == Work::kMemset) cleared.insert(w.at);
+            if (w.kind != Work::kLaunch || !w.launch.is("k_diag_gradients")) continue;
+            const lbm::DiagArgs& a = w.launch.as<lbm::DiagArgs>();
+            auto live = [&](const void* p) {
+                cudaPointerAttributes t;
+                return cudaPointerGetAttributes(&t, p) == cudaSuccess && t.type == cudaMemoryTypeDevice;
+            };
+            scratch = scratch && live(a.fields) && live(a.partials) && live(a.grad_rows) && live(a.finished) &&
+                      g_other.count(a.out) && cleared.count(a.finished);
+        }
+        lbm_destroy(h);
+        std::printf("%d first %d launches %zu second %d scratch %d left %zu\n", k, first, failed ? launches : (size_t)0,
+                    second, scratch ? 1 : 0, g_device.size() + g_other.size());
+        if (!failed) return 0;
+    }
+}
+
+}  // namespace
+
+int main(int argc, char** argv)
+{
+    const std::string what = argc > 1 ? argv[1] : "";
+    g_arg_bytes = [](const std::string& kernel) {
+        const auto has = [&](const char* k) { return kernel.find(k) != std::string::npos; };
+        return has("k_step") && !has("staged") ? sizeof(lbm::StepArgs) : has("k_diag_gradients") ? sizeof(lbm::DiagArgs) : 0;
+    };
+    if (what == "record") return record_scratch(std::atoi(argv[2]));
+    std::printf("unknown check '%s'\n", what.c_str());
+    return 2;
+}

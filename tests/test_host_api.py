@@ -1,0 +1,47 @@
+"""The library's host code (allocation, launch and stream logic of the C ABI) on
+the CPU: its objects linked with the stand-in CUDA runtime of
+tests/host_runtime.cpp, which records the work and can fail a chosen call."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2605_14505_gb300 import build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    try:
+        nvcc = build.nvcc()
+    except RuntimeError as e:
+        pytest.skip(str(e))
+    build.build()
+    exe = str(tmp_path_factory.mktemp("host_api") / "host_api")
+    objs = [os.path.join(build.OBJDIR, os.path.basename(s)[:-3] + ".o") for s in build.sources()]
+    cmd = [nvcc] + build.ARCH + ["-O1", "-std=c++17", "-I" + build.CSRC, "-I" + os.path.join(build.ROOT, "include"),
+                                 "-cudart", "none", "-o", exe, os.path.join(HERE, "host_api.cu"),
+                                 os.path.join(HERE, "host_runtime.cpp")] + objs
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+    def run(*args):
+        r = subprocess.run([exe] + [str(a) for a in args], capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stdout + r.stderr
+        return r.stdout.strip().splitlines()
+
+    return run
+
+
+@pytest.mark.parametrize("fused", [0, 1])
+def test_a_record_after_a_failed_one_has_its_scratch(host, fused):
+    """Whichever allocation of the first record fails, that call says so and
+    launches nothing; the next one passes kernels live scratch with a cleared
+    block count, and nothing outlives the handle."""
+    lines = [line.split() for line in host("record", fused)]
+    assert len(lines) >= 6
+    for k, (_, _, first, _, launches, _, second, _, scratch, _, left) in enumerate(lines):
+        assert int(first) == (-2 if k < len(lines) - 1 else 0), lines[k]
+        assert launches == "0", lines[k]
+        assert (second, scratch, left) == ("0", "1", "0"), lines[k]
