@@ -1860,12 +1860,10 @@ struct lbm_batch_ctx {
     cudaStream_t vstream[8] = {};
     cudaEvent_t vjoin[8] = {};
     cudaEvent_t vfork = nullptr;
-    // per-instance driver: chain c runs instances chain_of[c] in order, each
-    // with its own single-lattice step kernel; streams and join events are
-    // created on first use
-    std::vector<std::vector<int>> chain_of;
-    // the same driver's rounds: instances that L2 holds together run all steps
-    // of a call before the next round's
+    // per-instance driver: instances, largest store first; rounds of those
+    // that L2 holds together, which run all steps of a call before the next
+    // round's; streams and join events, created as they are needed
+    std::vector<int> order;
     std::vector<std::vector<int>> rounds;
     std::vector<cudaStream_t> cstream;
     std::vector<cudaEvent_t> cjoin;
@@ -1894,7 +1892,8 @@ struct lbm_batch_ctx {
 namespace {
 
 constexpr int kBatchGraphSteps = 64;
-constexpr int kMaxChains = 128;   // graph branches of the per-instance driver
+constexpr int kMaxChains = 128;   // streams of the per-instance driver
+constexpr int kRecordChains = 8;  // and of a batch's records
 
 void batch_drop_graph(lbm_batch_ctx* b)
 {
@@ -2035,28 +2034,31 @@ cudaError_t batch_launch_step(lbm_batch_ctx* b, int odd, cudaStream_t s)
     return cudaSuccess;
 }
 
-// Per-instance driver: instances sorted by bytes per step, largest first,
-// dealt round-robin to min(count, kMaxChains) chains, so that the longest
-// chains start first and the chains carry similar work.
-cudaError_t batch_ensure_chains(lbm_batch_ctx* b)
+// Streams and join events of the per-instance driver, at least `count` of them;
+// after a failure those that are complete stay.
+cudaError_t batch_ensure_streams(lbm_batch_ctx* b, size_t count)
 {
-    if (!b->chain_of.empty()) return cudaSuccess;
-    const int n = (int)b->inst.size();
-    std::vector<int> order(n);
-    for (int i = 0; i < n; ++i) order[i] = i;
-    auto bytes = [&](int i) { return b->inst[i]->store_bytes; };
-    std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return bytes(a) > bytes(c); });
-    const int nc = n < kMaxChains ? n : kMaxChains;
-    b->chain_of.assign(nc, {});
-    for (int k = 0; k < n; ++k) b->chain_of[k % nc].push_back(order[k]);
-    b->cstream.assign(nc, nullptr);
-    b->cjoin.assign(nc, nullptr);
-    for (int c = 0; c < nc; ++c) {
-        cudaError_t e = cudaStreamCreateWithFlags(&b->cstream[c], cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->cjoin[c], cudaEventDisableTiming);
-        if (e != cudaSuccess) return e;
+    while (b->cjoin.size() < count) {
+        cudaStream_t s = nullptr;
+        cudaEvent_t done = nullptr;
+        cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+        if (e != cudaSuccess) {
+            if (s) cudaStreamDestroy(s);
+            return e;
+        }
+        b->cstream.push_back(s);
+        b->cjoin.push_back(done);
     }
     return cudaSuccess;
+}
+
+// Instances dealt to at most `most` chains.
+std::vector<std::vector<int>> deal_chains(const std::vector<int>& instances, size_t most)
+{
+    std::vector<std::vector<int>> chains(std::min(instances.size(), most));
+    for (size_t k = 0; k < instances.size(); ++k) chains[k % chains.size()].push_back(instances[k]);
+    return chains;
 }
 
 // Rounds of the per-instance driver: instances in order of size, as many to a
@@ -2072,6 +2074,7 @@ void batch_build_rounds(lbm_batch_ctx* b)
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
     std::stable_sort(order.begin(), order.end(),
                      [&](int a, int c) { return b->inst[a]->store_bytes > b->inst[c]->store_bytes; });
+    b->order = order;
     const size_t budget = b->inst[0]->l2_bytes / 4 * 3;
     size_t held = 0;
     for (int i : order) {
@@ -2106,14 +2109,6 @@ int batch_run_chains(lbm_batch_ctx* b, const std::vector<std::vector<int>>& chai
     return LBM_OK;
 }
 
-// Instances dealt to at most `most` chains.
-std::vector<std::vector<int>> deal_chains(const std::vector<int>& instances, size_t most)
-{
-    std::vector<std::vector<int>> chains(std::min(instances.size(), most));
-    for (size_t k = 0; k < instances.size(); ++k) chains[k % chains.size()].push_back(instances[k]);
-    return chains;
-}
-
 // A call of one step keeps nothing in L2 and runs all instances at once (the
 // sweep above in calls of 1 / 2 / 4 / 100 steps: 970 / 956 / 821 / 728 us a step;
 // 4 steps all at once 1007).
@@ -2121,12 +2116,14 @@ constexpr int64_t kRoundSteps = 2;
 
 int batch_step_instances(lbm_batch_ctx* b, int64_t nsteps)
 {
-    LBM_CUDA(batch_ensure_chains(b), "batch chain streams");
-    // lbm_step on the chain's stream: the instance's own graph replays, eager steps outside them
-    if (nsteps < kRoundSteps) return batch_run_chains(b, b->chain_of, [&](lbm_ctx* h) { return lbm_step(h, nsteps); });
+    const size_t most = std::min<size_t>(b->inst.size(), kMaxChains);
+    LBM_CUDA(batch_ensure_streams(b, most), "batch chain streams");
     batch_build_rounds(b);
+    // lbm_step on the chain's stream: the instance's own graph replays, eager steps outside them
+    if (nsteps < kRoundSteps)
+        return batch_run_chains(b, deal_chains(b->order, most), [&](lbm_ctx* h) { return lbm_step(h, nsteps); });
     for (const std::vector<int>& round : b->rounds) {
-        const int rc = batch_run_chains(b, deal_chains(round, b->chain_of.size()), [&](lbm_ctx* h) {
+        const int rc = batch_run_chains(b, deal_chains(round, most), [&](lbm_ctx* h) {
             if (round.size() == 1) h->l2 = L2Use::alone;
             const int r = lbm_step(h, nsteps);
             h->l2 = L2Use::shared;
@@ -2433,11 +2430,10 @@ int lbm_batch_diagnostics(lbm_batch b, lbm_diag* out)
     // every instance's kernels first, on several streams, then one wait (one
     // instance after the other with a wait each: 64 instances 3.3 ms)
     if (b->stream != nullptr) {
-        LBM_CUDA(batch_ensure_chains(b), "batch chain streams");
+        const size_t most = std::min<size_t>(b->inst.size(), kRecordChains);
+        LBM_CUDA(batch_ensure_streams(b, most), "batch chain streams");
         batch_build_rounds(b);
-        std::vector<int> order;
-        for (const std::vector<int>& round : b->rounds) order.insert(order.end(), round.begin(), round.end());
-        rc = batch_run_chains(b, deal_chains(order, std::min<size_t>(b->cstream.size(), 8)), enqueue_diagnostics);
+        rc = batch_run_chains(b, deal_chains(b->order, most), enqueue_diagnostics);
         if (rc) return rc;
     } else {
         for (lbm_ctx* h : b->inst)

@@ -70,6 +70,57 @@ int record_scratch(int fused)
     }
 }
 
+// A per-instance batch call of 12 lattices whose k-th allocation (streams and
+// events among them) fails, and the same call again. One line per k until no
+// call fails. `open`: streams whose launches of the failed call the batch's
+// stream was not made to wait for; `null`: launches of either call on no stream.
+int batch_calls(const std::string& call)
+{
+    for (int k = 0;; ++k) {
+        std::vector<lbm_params> ps;
+        for (int n : {32, 16, 24, 20, 16, 32, 24, 20, 16, 16, 40, 8}) {
+            lbm_params p;
+            lbm_params_from_physics(&p, n, n, n, LBM_D3Q19_D3Q7, LBM_GUO, 100.0, 1.0, 1.0, 0.04);
+            ps.push_back(p);
+        }
+        lbm_batch b = nullptr;
+        lbm_batch_create(&b, ps.data(), (int)ps.size());
+        lbm_batch_set_mode(b, LBM_BATCH_INSTANCES, 100);
+        lbm_batch_init_tgv(b, 1, 1e-3);
+        lbm_handle h = nullptr;
+        void* own = nullptr;
+        lbm_batch_instance(b, 0, &h);
+        lbm_get_stream(h, &own);
+        std::vector<lbm_diag> d(ps.size());
+        auto run = [&] { return call == "step" ? lbm_batch_step(b, 3) : lbm_batch_diagnostics(b, d.data()); };
+        g_work.clear();
+        g_fail_in = k;
+        const int first = run();
+        const bool failed = g_fail_in < 0;
+        g_fail_in = -1;
+        std::map<cudaStream_t, bool> joined;
+        std::map<void*, cudaStream_t> recorded;
+        for (const Work& w : g_work) {
+            if (w.kind == Work::kLaunch && w.stream != own) joined[w.stream] = false;
+            if (w.kind == Work::kRecord) recorded[w.at] = w.stream;
+            if (w.kind == Work::kWait && w.stream == own) joined[recorded[w.at]] = true;
+        }
+        int open = 0;
+        for (const auto& j : joined) open += !j.second;
+        const int second = run();
+        int null = 0;
+        std::set<cudaStream_t> used;
+        for (const Work& w : g_work) {
+            null += w.kind == Work::kLaunch && w.stream == nullptr;
+            if (w.kind == Work::kLaunch) used.insert(w.stream);
+        }
+        lbm_batch_destroy(b);
+        std::printf("%d first %d open %d second %d null %d streams %zu left %zu\n", k, first, open, second, null,
+                    used.size(), g_device.size() + g_other.size());
+        if (!failed) return 0;
+    }
+}
+
 }  // namespace
 
 int main(int argc, char** argv)
@@ -80,6 +131,7 @@ int main(int argc, char** argv)
         return has("k_step") && !has("staged") ? sizeof(lbm::StepArgs) : has("k_diag_gradients") ? sizeof(lbm::DiagArgs) : 0;
     };
     if (what == "record") return record_scratch(std::atoi(argv[2]));
+    if (what == "batch") return batch_calls(argv[2]);
     std::printf("unknown check '%s'\n", what.c_str());
     return 2;
 }

@@ -45,3 +45,18 @@ def test_a_record_after_a_failed_one_has_its_scratch(host, fused):
         assert int(first) == (-2 if k < len(lines) - 1 else 0), lines[k]
         assert launches == "0", lines[k]
         assert (second, scratch, left) == ("0", "1", "0"), lines[k]
+
+
+@pytest.mark.parametrize("call", ["step", "record"])
+def test_a_batch_call_after_a_failed_one_runs_on_its_streams(host, call):
+    """Whichever stream, event or scratch of a per-instance batch call cannot be
+    had, that call fails and the next one runs every instance on a stream of
+    the batch; records take no more streams than they use."""
+    lines = [line.split() for line in host("batch", call)]
+    assert len(lines) >= 12
+    for k, (_, _, first, _, _, _, second, _, null, _, streams, _, left) in enumerate(lines):
+        assert (int(first) < 0) == (k < len(lines) - 1), lines[k]
+        assert (second, null, left) == ("0", "0", "0"), lines[k]
+    assert int(lines[-1][10]) == (12 if call == "step" else 8)
+    if call == "record":   # 8 streams and events, then each instance's scratch
+        assert [line[2] for line in lines[:17]] == ["-3"] * 16 + ["-2"]
