@@ -2089,24 +2089,25 @@ void batch_build_rounds(lbm_batch_ctx* b)
 }
 
 // work(h) for the instances of each chain with h on the chain's stream, the
-// chains forked from and joined back to b->stream.
+// chains forked from and joined back to b->stream, a chain whose work failed too.
 template <class Work>
 int batch_run_chains(lbm_batch_ctx* b, const std::vector<std::vector<int>>& chains, Work&& work)
 {
     LBM_CUDA(cudaEventRecord(b->vfork, b->stream), "batch fork");
-    for (size_t c = 0; c < chains.size(); ++c) {
+    int rc = LBM_OK;
+    for (size_t c = 0; c < chains.size() && rc == LBM_OK; ++c) {
         LBM_CUDA(cudaStreamWaitEvent(b->cstream[c], b->vfork, 0), "batch fork wait");
         for (int i : chains[c]) {
             lbm_ctx* h = b->inst[i];
             h->stream = b->cstream[c];
-            const int rc = work(h);
+            rc = work(h);
             h->stream = b->stream;
-            if (rc) return rc;
+            if (rc) break;
         }
         LBM_CUDA(cudaEventRecord(b->cjoin[c], b->cstream[c]), "batch join");
         LBM_CUDA(cudaStreamWaitEvent(b->stream, b->cjoin[c], 0), "batch join wait");
     }
-    return LBM_OK;
+    return rc;
 }
 
 // A call of one step keeps nothing in L2 and runs all instances at once (the

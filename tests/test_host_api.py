@@ -60,3 +60,12 @@ def test_a_batch_call_after_a_failed_one_runs_on_its_streams(host, call):
     assert int(lines[-1][10]) == (12 if call == "step" else 8)
     if call == "record":   # 8 streams and events, then each instance's scratch
         assert [line[2] for line in lines[:17]] == ["-3"] * 16 + ["-2"]
+
+
+@pytest.mark.parametrize("call", ["step", "record"])
+def test_a_failed_batch_call_leaves_no_chain_behind(host, call):
+    """Whatever the chains were given before a call failed, the batch's stream
+    waits for it: later work on that stream (another initialisation, a step, an
+    instance's own record) does not run beside it."""
+    for line in host("batch", call):
+        assert line.split()[4] == "0", line
