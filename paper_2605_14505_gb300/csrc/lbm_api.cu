@@ -1,5 +1,6 @@
 // C ABI (include/lbm.h): handle management, parameter mapping, launches,
 // CUDA-graph replay of the AA step pair, diagnostics, autotuning.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -842,9 +843,39 @@ int halo_slots(int q, int sign, int* slots)
     }
 }
 
-// LBM_OK if p is device memory of the handle's device (the halo copies are
-// device-to-device).
-int check_device_buffer(const lbm_ctx* h, const void* p)
+// Whether [p, p + bytes) is allocated device memory as far as the driver tells.
+// A range may span several mappings (a buffer in expandable memory).
+bool device_range(const void* p, size_t bytes)
+{
+    using Query = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Query query = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const cudaError_t e =
+            cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 3020, cudaEnableDefault, &found);
+        if (e != cudaSuccess || found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Query>(f);
+    }();
+    CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    for (bool first = true; bytes > 0; first = false) {
+        CUdeviceptr base = 0;
+        size_t size = 0;
+        if (!query || query(&base, &size, at) != CUDA_SUCCESS) return first;   // memory without an extent of its own
+        const size_t here = (size_t)(base + size - at);
+        if (here == 0) return false;
+        if (here >= bytes) return true;
+        at += here;
+        bytes -= here;
+    }
+    return true;
+}
+
+// LBM_OK if p is `bytes` of device memory on the handle's device. The halo
+// kernel takes the buffers as they are, so their extent is looked at here.
+int check_device_buffer(const lbm_ctx* h, const void* p, size_t bytes)
 {
     cudaPointerAttributes attr;
     cudaError_t e = cudaPointerGetAttributes(&attr, p);
@@ -852,6 +883,8 @@ int check_device_buffer(const lbm_ctx* h, const void* p)
         cudaGetLastError();
         return fail(LBM_EINVAL, "halo buffers must be device memory on the handle's device");
     }
+    if (!device_range(p, bytes))
+        return fail(LBM_EINVAL, "a halo buffer is shorter than the %zu bytes of lbm_halo_bytes", bytes);
     return LBM_OK;
 }
 
@@ -1661,7 +1694,9 @@ int lbm_halo_pack(lbm_handle h, int phase, void* to_lower, void* to_upper)
     if (!h->store) return fail(LBM_ESTATE, "halo exchange before the store exists");
     if (phase != 0 && phase != 1) return fail(LBM_EINVAL, "phase must be 0 (before an odd step) or 1 (after it)");
     if (!to_lower || !to_upper) return fail(LBM_EINVAL, "null buffer");
-    if ((rc = check_device_buffer(h, to_lower)) || (rc = check_device_buffer(h, to_upper))) return rc;
+    size_t bytes = 0;
+    lbm_halo_bytes(h, &bytes);
+    if ((rc = check_device_buffer(h, to_lower, bytes)) || (rc = check_device_buffer(h, to_upper, bytes))) return rc;
     const int top = h->p.nz - 1;
     // phase 0: own boundary planes (plane 1: e_z = +1 slots; plane nz-2: e_z = -1)
     // phase 1: ghost planes (plane 0: e_z = -1 slots; plane nz-1: e_z = +1)
@@ -1677,7 +1712,10 @@ int lbm_halo_unpack(lbm_handle h, int phase, const void* from_lower, const void*
     if (!h->store) return fail(LBM_ESTATE, "halo exchange before the store exists");
     if (phase != 0 && phase != 1) return fail(LBM_EINVAL, "phase must be 0 (before an odd step) or 1 (after it)");
     if (!from_lower || !from_upper) return fail(LBM_EINVAL, "null buffer");
-    if ((rc = check_device_buffer(h, from_lower)) || (rc = check_device_buffer(h, from_upper))) return rc;
+    size_t bytes = 0;
+    lbm_halo_bytes(h, &bytes);
+    if ((rc = check_device_buffer(h, from_lower, bytes)) || (rc = check_device_buffer(h, from_upper, bytes)))
+        return rc;
     const int top = h->p.nz - 1;
     // phase 0: into the ghost planes (plane 0: e_z = -1 slots; plane nz-1: e_z = +1)
     // phase 1: into the own boundary planes (plane 1: e_z = +1; plane nz-2: e_z = -1)

@@ -121,6 +121,33 @@ int batch_calls(const std::string& call)
     }
 }
 
+// Pack and unpack with buffers that end `short_by` bytes before lbm_halo_bytes,
+// one of the two at a time: statuses and launches.
+int halo_buffers(long short_by)
+{
+    lbm_handle h = make(33, 9, 6, LBM_D3Q27_D3Q19, LBM_FP16_DEV);
+    start(h);
+    lbm_set_slab(h, 1);
+    size_t bytes = 0;
+    lbm_halo_bytes(h, &bytes);
+    void *whole = nullptr, *cut = nullptr;
+    cudaMalloc(&whole, bytes + 64);
+    cudaMalloc(&cut, bytes + 64);
+    char* w = static_cast<char*>(whole) + 64;
+    char* c = static_cast<char*>(cut) + 64 + short_by;
+    for (int phase = 0; phase < 2; ++phase)
+        for (int side = 0; side < 2; ++side) {
+            g_work.clear();
+            const int p = lbm_halo_pack(h, phase, side ? w : c, side ? c : w);
+            const int u = lbm_halo_unpack(h, phase, side ? w : c, side ? c : w);
+            std::printf("pack %d unpack %d launches %zu\n", p, u, g_work.size());
+        }
+    cudaFree(whole);
+    cudaFree(cut);
+    lbm_destroy(h);
+    return 0;
+}
+
 }  // namespace
 
 int main(int argc, char** argv)
@@ -132,6 +159,7 @@ int main(int argc, char** argv)
     };
     if (what == "record") return record_scratch(std::atoi(argv[2]));
     if (what == "batch") return batch_calls(argv[2]);
+    if (what == "halo") return halo_buffers(std::atol(argv[2]));
     std::printf("unknown check '%s'\n", what.c_str());
     return 2;
 }

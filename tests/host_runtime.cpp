@@ -4,6 +4,8 @@
 // Device: 152 SMs, 129 MiB of L2.
 #include "host_runtime.h"
 
+#include <cuda.h>
+
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -106,6 +108,24 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* n, const void*, i
 cudaError_t cudaGetSymbolAddress(void** p, const void*)
 {
     *p = reinterpret_cast<void*>(0x6000000000ull);
+    return cudaSuccess;
+}
+static CUresult address_range(CUdeviceptr* base, size_t* size, CUdeviceptr p)
+{
+    auto it = g_device.upper_bound(reinterpret_cast<char*>(p));
+    if (it == g_device.begin()) return CUDA_ERROR_NOT_FOUND;
+    --it;
+    if (reinterpret_cast<char*>(p) >= it->first + it->second) return CUDA_ERROR_NOT_FOUND;
+    *base = reinterpret_cast<CUdeviceptr>(it->first);
+    *size = it->second;
+    return CUDA_SUCCESS;
+}
+cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** f, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult* found)
+{
+    const bool known = std::strcmp(name, "cuMemGetAddressRange") == 0;
+    *f = known ? reinterpret_cast<void*>(address_range) : nullptr;
+    if (found) *found = known ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
     return cudaSuccess;
 }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p)

@@ -69,3 +69,10 @@ def test_a_failed_batch_call_leaves_no_chain_behind(host, call):
     instance's own record) does not run beside it."""
     for line in host("batch", call):
         assert line.split()[4] == "0", line
+
+
+@pytest.mark.parametrize("short_by,status,launches", [(-64, 0, 2), (0, 0, 2), (1, -1, 0), (5000, -1, 0)])
+def test_halo_buffers_are_as_long_as_said(host, short_by, status, launches):
+    """A buffer that ends at its last byte is taken, one that ends before it is
+    refused with nothing launched."""
+    assert host("halo", short_by) == [f"pack {status} unpack {status} launches {launches}"] * 4
