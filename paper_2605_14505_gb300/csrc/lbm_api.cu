@@ -113,7 +113,7 @@ struct lbm_ctx {
     double* diag_partials = nullptr;
     int diag_rows = 0;                 // rows of kDNumSlots the partials hold
     cudaEvent_t diag_event = nullptr;  // diagnostics copied to the host
-    float2* diag_grad = nullptr;       // pass-2 rows, then the count of finished blocks
+    double* diag_grad = nullptr;       // pass-2 rows, then the count of finished blocks
     double* diag_host = nullptr;       // pinned; the totals, written by the last kernel itself
     // host<->device staging
     double* staging = nullptr;
@@ -334,12 +334,14 @@ uint32_t moment_blocks(const lbm_ctx* h, uint32_t nodes)
     return std::min(4u * (uint32_t)h->num_sms, (nodes + kDiagBlock - 1) / kDiagBlock);
 }
 
-// Pass 2: planes per thread, at most 16 (the march's three loads ahead are
-// paid once per run) and few enough for 8 blocks per SM.
+// Pass 2: planes per thread, at most 32 and few enough for 6 blocks per SM. A
+// run pays for the march's three loads ahead and for its block's FP64 sums once:
+// records of D3Q27xD3Q19 at 128^3 98 us (104 with runs for 8 blocks per SM), at
+// 256^3 605 (614 with at most 16 planes), of D3Q19xD3Q7 at 384^3 1324 (1360).
 dim3 gradient_grid(const lbm_ctx* h, int& planes)
 {
     const int64_t bx = ((int64_t)h->p.nx * h->p.ny + kDiagBlock - 1) / kDiagBlock;
-    planes = (int)std::min<int64_t>(16, std::max<int64_t>(1, bx * h->p.nz / (8 * (int64_t)h->num_sms)));
+    planes = (int)std::min<int64_t>(32, std::max<int64_t>(1, bx * h->p.nz / (6 * (int64_t)h->num_sms)));
     return dim3((unsigned)bx, (unsigned)((h->p.nz + planes - 1) / planes));
 }
 
@@ -350,14 +352,14 @@ int ensure_diag(lbm_ctx* h, int rows)
     if (!h->diag_event) {   // the handle gets all of it or, where a part fails, nothing
         int planes = 0;
         const dim3 g = gradient_grid(h, planes);
-        const size_t pairs = (size_t)g.x * g.y * kDiagPass2;
+        const size_t sums = (size_t)g.x * g.y * kDiagPass2;
         float* fields = nullptr;
-        float2* grad = nullptr;
+        double* grad = nullptr;
         double* host = nullptr;
         cudaEvent_t event = nullptr;
         if (cudaMalloc(&fields, 4 * (size_t)h->geo.n3 * sizeof(float)) != cudaSuccess ||
-            cudaMalloc(&grad, (pairs + 1) * sizeof(float2)) != cudaSuccess ||
-            cudaMemsetAsync(grad + pairs, 0, sizeof(float2), h->stream) != cudaSuccess ||
+            cudaMalloc(&grad, (sums + 1) * sizeof(double)) != cudaSuccess ||
+            cudaMemsetAsync(grad + sums, 0, sizeof(double), h->stream) != cudaSuccess ||
             cudaMallocHost(&host, 16 * sizeof(double)) != cudaSuccess ||
             cudaEventCreateWithFlags(&event, cudaEventDisableTiming) != cudaSuccess) {
             cudaGetLastError();
@@ -735,8 +737,8 @@ cudaError_t step_skewed(lbm_ctx* h, const SkewPlan& p, int64_t nsteps, cudaStrea
 
 // What follows pass 1, whose `rows` rows are in h->diag_partials: more than
 // kDirectRows of them are first added up on every SM (into the rows behind
-// them), then pass 2 adds up what is left with its own rows and writes the
-// totals; a z-slab has no pass 2.
+// them), then pass 2 totals what is left beside its own sums; a z-slab has no
+// pass 2.
 constexpr int kDirectRows = 1024;
 cudaError_t launch_totals(lbm_ctx* h, DiagArgs a, int rows)
 {
@@ -752,11 +754,12 @@ cudaError_t launch_totals(lbm_ctx* h, DiagArgs a, int rows)
     }
     if (h->slab) {
         void* args[] = {&at, &rows, &a.out};
-        return launch_overlapped(diag_rows_kernel(), dim3(1), dim3(kDiagBlock), args, h->stream);
+        return launch_overlapped(diag_totals_kernel(), dim3(kDiagPass1), dim3(kDiagBlock), args, h->stream);
     }
     a.partials = at;
     a.rows = rows;
-    const dim3 grid = gradient_grid(h, a.planes);
+    dim3 grid = gradient_grid(h, a.planes);
+    grid.y += (kDiagPass1 + grid.x - 1) / grid.x;   // the blocks that total the pass-1 slots
     void* args[] = {&a};
     return launch_overlapped(diag_gradients_kernel(), grid, dim3(kDiagBlock), args, h->stream);
 }
@@ -1825,7 +1828,7 @@ int lbm_diagnostics_noalloc(lbm_handle h, lbm_diag* out)
     int nb = (int)blocks;
     double* dout = scratch + kStaticOutOffset;
     void* fargs[] = {&pp, &nb, &dout};
-    LBM_CUDA(cudaLaunchKernel(diag_rows_kernel(), dim3(1), dim3(kDiagBlock), fargs, 0, h->stream),
+    LBM_CUDA(cudaLaunchKernel(diag_totals_kernel(), dim3(kDiagPass1), dim3(kDiagBlock), fargs, 0, h->stream),
              "static diag pass 2");
     double s[kDiagPass1];
     LBM_CUDA(cudaMemcpyAsync(s, dout, sizeof(s), cudaMemcpyDeviceToHost, h->stream), "static diag copy");

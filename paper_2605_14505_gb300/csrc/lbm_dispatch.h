@@ -29,6 +29,7 @@ const KernelSet* kernel_set(int pair, int storage);
 
 const void* diag_gradients_kernel();
 const void* diag_rows_kernel();
+const void* diag_totals_kernel();
 
 // Batched update (FP32 storage, D3Q27xD3Q19 and D3Q19xD3Q7, all forcings).
 const void* batch_variant_kernel(int variant, int odd);   // variant = 4 * pair + forcing

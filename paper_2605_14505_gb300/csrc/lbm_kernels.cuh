@@ -35,10 +35,20 @@ struct DiagArgs {
     // pass 2, whose last block sums everything
     int planes;          // planes a thread marches through
     int rows;            // pass-1 rows
-    float2* grad_rows;   // kDiagPass2 pairs per block
+    double* grad_rows;   // kDiagPass2 sums per block
     unsigned* finished;  // blocks done; 0 between launches
     double* out;         // kDNumSlots totals
 };
+
+// x as FP64, zeros and normal numbers by integer operations: the conversion
+// instruction runs at the FP64 pipe's rate (16 cycles for a warp's).
+__device__ __forceinline__ double widen(float x)
+{
+    const uint32_t u = __float_as_uint(x), sign = u & 0x80000000u, m = u & 0x7fffffffu;
+    if (m == 0u) return __hiloint2double((int)sign, 0);
+    if (m - 0x00800000u >= 0x7f000000u) return (double)x;
+    return __hiloint2double((int)(sign | ((m >> 3) + (896u << 20))), (int)(m << 29));
+}
 
 // Compensated (Kahan) FP32 running sum for a thread's share of a diagnostics
 // reduction: within a few FP32 ulps of the exact sum of its terms, on the FP32
@@ -53,6 +63,7 @@ struct KahanF {
         c = (t - s) - y;
         s = t;
     }
+    __device__ __forceinline__ double value() const { return widen(s) - widen(c); }
 };
 
 // What a kernel needs to add one node's diagnostics (pass 1): the scales of
@@ -114,6 +125,52 @@ __device__ __forceinline__ float2 block_sum_pairs(float (&hi)[N], float (&lo)[N]
     float2 v = sh[0][tid];
     for (int w = 1; w < nwarps; ++w) add(tid == MAXQ, v.x, v.y, sh[w][tid].x, sh[w][tid].y);
     return v;
+}
+
+// The same of FP64 values, for blocks of kDiagBlock threads in a row. A warp
+// halves the values with its lanes (a lane that differs in bit o gives the
+// other half of what is left and keeps its own), so two values take 5 FP64 adds
+// of a warp instead of 10: this GPU's FP64 pipe takes 16 cycles for each. A warp
+// per value behind shared memory needs fewer still, but in a chain: the 32^3
+// record of k_diag_gradients 22.5 us against 21.0.
+template <int N, int MAXQ>
+__device__ __forceinline__ double block_sum(double (&v)[N])
+{
+    static_assert(N <= 4, "the last step takes four values");
+    constexpr int kWarps = kDiagBlock / 32;
+    __shared__ double sh[kWarps][N];
+    const int lane = (int)threadIdx.x & 31, wid = (int)threadIdx.x >> 5;
+    int q0 = 0, q1 = N;   // the values this lane holds, v[0] being q0's
+    int left = N;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = (lane & o) != 0 && left > 1;
+        const int half = (left + 1) / 2;
+        if (up)
+            q0 += half;
+        else if (left > 1)
+            q1 = min(q1, q0 + half);
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const double far = i + half < left ? v[i + half] : 0.0;
+            const double mine = up ? far : v[i];
+            const double got = __shfl_xor_sync(0xffffffffu, up || left == 1 ? v[i] : far, o);
+            v[i] = q0 + i == MAXQ ? fmax(mine, got) : mine + got;
+        }
+        left = half;
+    }
+    if (q0 < q1) sh[wid][q0] = v[0];
+    __syncthreads();
+    if (wid > 0) return 0.0;
+    // value lane / 8 of warp lane % 8's; value q to thread q
+    const int q = lane / kWarps;
+    double sum = q < N ? sh[lane % kWarps][q] : 0.0;
+#pragma unroll
+    for (int o = kWarps / 2; o > 0; o >>= 1) {
+        const double got = __shfl_xor_sync(0xffffffffu, sum, o);
+        sum = q == MAXQ ? fmax(sum, got) : sum + got;
+    }
+    return __shfl_sync(0xffffffffu, sum, kWarps * (lane % 4));
 }
 
 struct DiagAcc {
@@ -192,6 +249,25 @@ __device__ __forceinline__ void add_rows(const double* rows, int first, int last
             }
         }
     }
+}
+
+// Total of slot q of the rows, in thread 0: pairs in a thread, FP64 across threads.
+__device__ __forceinline__ double sum_slot(const double* rows, int nb, int q)
+{
+    float hi = 0.f, lo = 0.f;
+    for (int b = (int)threadIdx.x; b < nb; b += kDiagBlock) {
+        const float2 v = reinterpret_cast<const float2*>(rows + (size_t)b * kDNumSlots)[q];
+        if (q == kDUmax) {
+            hi = fmaxf(hi, v.x);
+        } else {
+            float t, e;
+            two_sum(hi, v.x, t, e);
+            hi = t;
+            lo = lo + v.y + e;
+        }
+    }
+    double v[1] = {widen(hi) + widen(lo)};
+    return q == kDUmax ? block_sum<1, 0>(v) : block_sum<1, -1>(v);
 }
 
 // One node's pass-1 diagnostics from its post-stream, pre-collision
@@ -1129,9 +1205,11 @@ __global__ void __launch_bounds__(kDiagBlock, P::QF + P::QG > 46 ? 3 : 4) k_diag
 // through a.planes planes with rho', ux, uy of three planes in registers: 15
 // loads and no division per node, against 18 loads and two divisions with a
 // strided loop over the nodes (0.091 against 0.130 ms at 256^3, where the 16 B
-// per node take 0.040; what is left is load issue). The last block to finish adds all pass-1 and pass-2 rows in
-// a fixed order and writes the totals to pinned memory, so neither a launch nor
-// a copy follows: one fused step and its record at 32^3 21 us against 45.
+// per node take 0.040; what is left is load issue). Beyond a thread's own sums
+// all is FP64. The first rows of blocks total a pass-1 slot each, and the last
+// of the others to finish adds all pass-2 rows in a fixed order; both write to
+// pinned memory, so neither a launch nor a copy follows: one fused step and its
+// record at 32^3 21.0 us against 45. With all slots in the last block it took 25.
 __global__ void __launch_bounds__(kDiagBlock, 4) k_diag_gradients(DiagArgs a)
 {
     const uint32_t nx = (uint32_t)a.geo.nx, ny = (uint32_t)a.geo.ny, nz = (uint32_t)a.geo.nz, nxy = nx * ny;
@@ -1141,10 +1219,20 @@ __global__ void __launch_bounds__(kDiagBlock, 4) k_diag_gradients(DiagArgs a)
     const float* uy = a.fields + 2 * n3;
     const float* uz = a.fields + 3 * n3;
     const uint32_t r = blockIdx.x * kDiagBlock + threadIdx.x;
-    const uint32_t z0 = blockIdx.y * (uint32_t)a.planes;
+    const uint32_t slot_rows = (kDiagPass1 + gridDim.x - 1) / gridDim.x;
+    wait_prerequisites();
+    if (blockIdx.y < slot_rows) {
+        const uint32_t q = blockIdx.x + gridDim.x * blockIdx.y;
+        if (q >= kDiagPass1) return;
+        const double sum = sum_slot(a.partials, a.rows, (int)q);
+        if (threadIdx.x == 0) a.out[q] = sum;
+        return;
+    }
+    const uint32_t run = blockIdx.y - slot_rows, blocks = gridDim.x * (gridDim.y - slot_rows);
+    const uint32_t block = blockIdx.x + gridDim.x * run;
+    const uint32_t z0 = run * (uint32_t)a.planes;
     const uint32_t z1 = min(z0 + (uint32_t)a.planes, nz);
     KahanF acc[kDiagPass2];
-    wait_prerequisites();
     if (r < nxy) {
         const uint32_t y = r / nx, x = r - y * nx;
         const uint32_t xm = x == 0 ? r + nx - 1 : r - 1, xp = x == nx - 1 ? r - x : r + 1;
@@ -1174,11 +1262,10 @@ __global__ void __launch_bounds__(kDiagBlock, 4) k_diag_gradients(DiagArgs a)
         }
     }
     launch_dependents();
-    const uint32_t block = blockIdx.x + gridDim.x * blockIdx.y, blocks = gridDim.x * gridDim.y;
     {
-        float hi[kDiagPass2] = {acc[0].s, acc[1].s}, lo[kDiagPass2] = {-acc[0].c, -acc[1].c};
-        const float2 v = block_sum_pairs<kDiagPass2, -1>(hi, lo);
-        if (threadIdx.x < kDiagPass2) a.grad_rows[(size_t)block * kDiagPass2 + threadIdx.x] = v;
+        double v[kDiagPass2] = {acc[0].value(), acc[1].value()};
+        const double sum = block_sum<kDiagPass2, -1>(v);
+        if (threadIdx.x < kDiagPass2) a.grad_rows[(size_t)block * kDiagPass2 + threadIdx.x] = sum;
     }
     __shared__ bool last;
     if (threadIdx.x < 32) {   // the warp that wrote the row
@@ -1189,27 +1276,19 @@ __global__ void __launch_bounds__(kDiagBlock, 4) k_diag_gradients(DiagArgs a)
     __syncthreads();
     if (!last) return;
     __threadfence();
-    float hi[kDNumSlots] = {}, lo[kDNumSlots] = {};
-    add_rows(a.partials, 0, a.rows, hi, lo);
+    double v[kDiagPass2] = {};
     for (uint32_t b = threadIdx.x; b < blocks; b += kDiagBlock) {
 #pragma unroll
-        for (int q = 0; q < kDiagPass2; ++q) {
-            const float2 v = __ldcg(a.grad_rows + (size_t)b * kDiagPass2 + q);
-            float t, e;
-            two_sum(hi[kDiagPass1 + q], v.x, t, e);
-            hi[kDiagPass1 + q] = t;
-            lo[kDiagPass1 + q] += v.y + e;
-        }
+        for (int q = 0; q < kDiagPass2; ++q) v[q] += __ldcg(a.grad_rows + (size_t)b * kDiagPass2 + q);
     }
-    const float2 v = block_sum_pairs<kDNumSlots, kDUmax>(hi, lo);
-    if (threadIdx.x < kDNumSlots) a.out[threadIdx.x] = (double)v.x + (double)v.y;
+    const double sum = block_sum<kDiagPass2, -1>(v);
+    if (threadIdx.x < kDiagPass2) a.out[kDiagPass1 + threadIdx.x] = sum;
     if (threadIdx.x == 0) *a.finished = 0u;
 }
 
-// Pass-1 rows added up: block b of the grid sums its contiguous share of the
-// nb rows. With one block the totals go to out[0..kDiagPass1) as FP64; with
-// more (a step kernel's row per block, 65536 rows at 256^3, spread over the
-// SMs before k_diag_gradients reads them) each block writes its row of out.
+// More pass-1 rows than are added up directly (a step kernel's row per block,
+// 65536 rows at 256^3), spread over the SMs: block b of the grid sums its
+// contiguous share of the nb rows into row b of out.
 __global__ void __launch_bounds__(kDiagBlock) k_diag_rows(const double* rows, int nb, double* out)
 {
     wait_prerequisites();
@@ -1219,11 +1298,17 @@ __global__ void __launch_bounds__(kDiagBlock) k_diag_rows(const double* rows, in
     float hi[kDiagPass1] = {}, lo[kDiagPass1] = {};
     add_rows(rows, first, last, hi, lo);
     const float2 v = block_sum_pairs<kDiagPass1, kDUmax>(hi, lo);
-    if (threadIdx.x >= kDiagPass1) return;
-    if (gridDim.x > 1)
+    if (threadIdx.x < kDiagPass1)
         reinterpret_cast<float2*>(out + (size_t)blockIdx.x * kDNumSlots)[threadIdx.x] = v;
-    else
-        out[threadIdx.x] = (double)v.x + (double)v.y;
+}
+
+// Totals of pass 1 where no pass 2 follows, a block per slot.
+__global__ void __launch_bounds__(kDiagBlock) k_diag_totals(const double* rows, int nb, double* out)
+{
+    wait_prerequisites();
+    launch_dependents();
+    const double sum = sum_slot(rows, nb, (int)blockIdx.x);
+    if (threadIdx.x == 0) out[blockIdx.x] = sum;
 }
 
 #endif  // LBM_REDUCTION_KERNELS

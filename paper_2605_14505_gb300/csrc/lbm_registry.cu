@@ -42,5 +42,6 @@ const KernelSet* kernel_set(int pair, int storage)
 
 const void* diag_gradients_kernel() { return (const void*)k_diag_gradients; }
 const void* diag_rows_kernel() { return (const void*)k_diag_rows; }
+const void* diag_totals_kernel() { return (const void*)k_diag_totals; }
 
 }  // namespace lbm
