@@ -29,10 +29,10 @@
 namespace lbm {
 
 // One node of one instance: identical arithmetic to k_step.
-template <class P, int FORCING, bool ODD>
+template <class P, int FORCING, bool ODD, int REUSE>
 __device__ __forceinline__ void batch_node(const BatchInstance& I, int x, int y, int z)
 {
-    update_node<P, FORCING, float, ODD>(I.f, I.g, I.geo, I.ph, x, y, z);
+    update_node<P, FORCING, float, ODD, REUSE>(I.f, I.g, I.geo, I.ph, x, y, z);
 }
 
 // Tile t of the global list: its instance and this thread's node; false if
@@ -51,34 +51,23 @@ __device__ __forceinline__ bool tile_node(const BatchArgs& A, uint32_t t, const 
     return x < I.geo.nx && y < I.geo.ny;
 }
 
-template <bool ODD>
-__device__ __forceinline__ void batch_tile(const BatchArgs& A, uint32_t t)
-{
-    const BatchInstance* I;
-    int x, y, z;
-    if (!tile_node(A, t, I, x, y, z)) return;
-    switch (I->variant) {
-    case 0: batch_node<Pair<27, 19>, kGuo, ODD>(*I, x, y, z); break;
-    case 1: batch_node<Pair<27, 19>, kShanChen, ODD>(*I, x, y, z); break;
-    case 2: batch_node<Pair<27, 19>, kEDM, ODD>(*I, x, y, z); break;
-    case 3: batch_node<Pair<27, 19>, kHCZ, ODD>(*I, x, y, z); break;
-    case 4: batch_node<Pair<19, 7>, kGuo, ODD>(*I, x, y, z); break;
-    case 5: batch_node<Pair<19, 7>, kShanChen, ODD>(*I, x, y, z); break;
-    case 6: batch_node<Pair<19, 7>, kEDM, ODD>(*I, x, y, z); break;
-    default: batch_node<Pair<19, 7>, kHCZ, ODD>(*I, x, y, z); break;
-    }
-}
-
 // Per-step driver: one launch per (pair, forcing) variant over that variant's
 // tiles, which the host lists contiguously. Without the other variants'
-// code the kernel fits three 256-thread blocks per SM, as k_step does.
+// code the kernel fits three 256-thread blocks per SM, as k_step does. Every
+// launch passes one way over its instances, so their populations are
+// evict-first: 1012 us a step of the 64-lattice sweep (32^3 to 96^3, both pairs,
+// four Froude numbers, Guo and Shan-Chen) against 1047 with the normal priority
+// of k_step, 524 against 553 for EDM and HCZ, four 96^3 213.6 against 225.5. The
+// persistent kernel runs a large instance's consecutive steps closer together
+// and is better off with the normal priority (four 96^3 209.2 against 210.9, six
+// of 50^3 and 70^3 94 either way, the sweep 966.5 against 968).
 template <class P, int FORCING, bool ODD>
 __global__ void __launch_bounds__(256, 3) k_batch_variant(BatchArgs A)
 {
     for (uint32_t t = A.tile_begin + blockIdx.x; t < A.tile_end; t += gridDim.x) {
         const BatchInstance* I;
         int x, y, z;
-        if (tile_node(A, t, I, x, y, z)) batch_node<P, FORCING, ODD>(*I, x, y, z);
+        if (tile_node(A, t, I, x, y, z)) batch_node<P, FORCING, ODD, kOnce>(*I, x, y, z);
     }
 }
 
@@ -97,7 +86,7 @@ __device__ __forceinline__ void flow_nodes(const BatchInstance& I, uint32_t n0, 
     const int nx = I.geo.nx, ny = I.geo.ny;
     const int dy = (int)(blockDim.x / (unsigned)nx), dx = (int)blockDim.x - dy * nx;
     for (; n < n1; n += blockDim.x) {
-        batch_node<P, FORCING, ODD>(I, x, y, z);
+        batch_node<P, FORCING, ODD, kKeep>(I, x, y, z);
         x += dx;
         y += dy;
         if (x >= nx) {

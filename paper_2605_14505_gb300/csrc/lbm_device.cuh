@@ -120,7 +120,10 @@ LBM_HD void sfor(F&& f)
 // ---------------------------------------------------------------------------
 // Storage codec (round to nearest even on store).
 // ---------------------------------------------------------------------------
-template <class T>
+// What a kernel's populations are worth in L2: to be kept for the next step, or
+// read and written once.
+enum Reuse : int { kKeep = 0, kOnce = 1 };
+template <class T, int REUSE = kKeep>
 __device__ __forceinline__ float ld_pop(const T* p);
 // Population loads ask L2 to fetch the whole 256-byte block around the address.
 // A warp's row segment is 128 bytes in FP32 (64 in 16-bit storage) and the next
@@ -128,8 +131,9 @@ __device__ __forceinline__ float ld_pop(const T* p);
 // stores keep the normal priority in L2: the next step starts where this one
 // ends and finds it there (as evict-first, `.cs`, 96^3 D3Q27xD3Q19 FP32 42.7
 // against 42.5 us per step, 256^3 898 against 894, D3Q19xD3Q7 509.5 against
-// 507.9). The block lies in the same mapped page as the address, so the hint
-// never reaches past the allocation's pages.
+// 507.9). kOnce, for a kernel that passes one way over more than L2 holds, is
+// that evict-first form (FP32). The block lies in the same mapped page as the
+// address, so the hint never reaches past the allocation's pages.
 __device__ __forceinline__ uint16_t ld_u16(const void* p)
 {
     uint16_t v;
@@ -153,10 +157,19 @@ __device__ __forceinline__ float ld_pop<__nv_bfloat16>(const __nv_bfloat16* p)
 {
     return __bfloat162float(__ushort_as_bfloat16(ld_u16(p)));
 }
-template <class T>
+template <>
+__device__ __forceinline__ float ld_pop<float, kOnce>(const float* p)
+{
+    float v;
+    asm volatile("ld.global.cs.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+template <class T, int REUSE = kKeep>
 __device__ __forceinline__ void st_pop(T* p, float v);
 template <>
 __device__ __forceinline__ void st_pop<float>(float* p, float v) { *p = v; }
+template <>
+__device__ __forceinline__ void st_pop<float, kOnce>(float* p, float v) { __stcs(p, v); }
 template <>
 __device__ __forceinline__ void st_pop<__half>(__half* p, float v) { *p = __float2half_rn(v); }
 template <>
@@ -303,7 +316,7 @@ struct AA {
 #ifndef LBM_ADDR64
 #define LBM_ADDR64 0
 #endif
-template <class L, bool ODD, class T>
+template <class L, bool ODD, class T, int REUSE = kKeep>
 __device__ __forceinline__ void load_node(const T* __restrict__ base, uint32_t n3, const NodeAddr& a,
                                           float* v)
 {
@@ -311,15 +324,15 @@ __device__ __forceinline__ void load_node(const T* __restrict__ base, uint32_t n
         constexpr int i = decltype(ic)::value;
 #if LBM_ADDR64
         const T* p = base + AA<L, ODD>::template read_off<i>(a);
-        v[i] = ld_pop<T>(p + (size_t)AA<L, ODD>::template read_slot<i>() * n3);
+        v[i] = ld_pop<T, REUSE>(p + (size_t)AA<L, ODD>::template read_slot<i>() * n3);
 #else
-        v[i] = ld_pop<T>(base + (AA<L, ODD>::template read_slot<i>() * n3 +
-                                 AA<L, ODD>::template read_off<i>(a)));
+        v[i] = ld_pop<T, REUSE>(base + (AA<L, ODD>::template read_slot<i>() * n3 +
+                                        AA<L, ODD>::template read_off<i>(a)));
 #endif
     });
 }
 
-template <class L, bool ODD, class T>
+template <class L, bool ODD, class T, int REUSE = kKeep>
 __device__ __forceinline__ void store_node(T* __restrict__ base, uint32_t n3, const NodeAddr& a,
                                            const float* v)
 {
@@ -327,11 +340,11 @@ __device__ __forceinline__ void store_node(T* __restrict__ base, uint32_t n3, co
         constexpr int i = decltype(ic)::value;
 #if LBM_ADDR64
         T* p = base + AA<L, ODD>::template write_off<i>(a);
-        st_pop<T>(p + (size_t)AA<L, ODD>::template write_slot<i>() * n3, v[i]);
+        st_pop<T, REUSE>(p + (size_t)AA<L, ODD>::template write_slot<i>() * n3, v[i]);
 #else
-        st_pop<T>(base + (AA<L, ODD>::template write_slot<i>() * n3 +
-                          AA<L, ODD>::template write_off<i>(a)),
-                  v[i]);
+        st_pop<T, REUSE>(base + (AA<L, ODD>::template write_slot<i>() * n3 +
+                                 AA<L, ODD>::template write_off<i>(a)),
+                         v[i]);
 #endif
     });
 }

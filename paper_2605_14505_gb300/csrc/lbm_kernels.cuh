@@ -419,7 +419,7 @@ struct SamePlace {
 // along x), moments, coupled rho'/u solve, f and g collisions, store.
 // hook(h, m) runs between the moments and the collisions (the diagnosing
 // step kernels read the pre-collision state there).
-template <class P, int FORCING, class T, bool ODD, class Hook, class Place = SamePlace>
+template <class P, int FORCING, class T, bool ODD, int REUSE = kKeep, class Hook, class Place = SamePlace>
 __device__ __forceinline__ void update_node(void* fv, void* gv, const Geometry& geo, const Phys& ph, int x,
                                             int y, int z, Hook&& hook, Place place = Place())
 {
@@ -429,20 +429,20 @@ __device__ __forceinline__ void update_node(void* fv, void* gv, const Geometry& 
     const uint32_t n3 = geo.n3;
     constexpr bool kExact = std::is_same<T, float>::value;
     float h[P::QF], k[P::QG];
-    load_node<typename P::LF, ODD, T>(f, n3, a, h);
-    load_node<typename P::LG, ODD, T>(g, n3, a, k);
+    load_node<typename P::LF, ODD, T, REUSE>(f, n3, a, h);
+    load_node<typename P::LG, ODD, T, REUSE>(g, n3, a, k);
     collide_node<P, FORCING, kExact>(h, k, ph, hook);
     place(x, y, z);
     const NodeAddr b = node_addr<T>(geo, x, y, z);
-    store_node<typename P::LF, ODD, T>(f, n3, b, h);
-    store_node<typename P::LG, ODD, T>(g, n3, b, k);
+    store_node<typename P::LF, ODD, T, REUSE>(f, n3, b, h);
+    store_node<typename P::LG, ODD, T, REUSE>(g, n3, b, k);
 }
 
-template <class P, int FORCING, class T, bool ODD>
+template <class P, int FORCING, class T, bool ODD, int REUSE = kKeep>
 __device__ __forceinline__ void update_node(void* fv, void* gv, const Geometry& geo, const Phys& ph, int x,
                                             int y, int z)
 {
-    update_node<P, FORCING, T, ODD>(fv, gv, geo, ph, x, y, z, [](const float*, const Macro&) {});
+    update_node<P, FORCING, T, ODD, REUSE>(fv, gv, geo, ph, x, y, z, [](const float*, const Macro&) {});
 }
 
 // Three 256-thread blocks per SM (<= 85 registers): measured on the 256^3
