@@ -186,6 +186,20 @@ double step_waves(const lbm_ctx* h)
 // Less than one wave of the longer kernels: every step is one block's latency.
 bool one_short_wave(const lbm_ctx* h) { return h->q.qf + h->q.qg >= 38 && step_waves(h) <= 1.0; }
 
+// Whether a step's blocks may wait on the SMs for the end of the step before
+// (launch_overlapped). Nearly always the faster: 64^3 FP32 D3Q27xD3Q19 11.7
+// against 12.2 us per step, 32^3 D3Q19xD3Q7 2.2 against 2.7, D3Q19xD3Q19 2.69
+// against 3.15, D3Q27xD3Q19 FP16 3.2 against 3.8 and at 20^3 3.1 against 3.6.
+// Not for the longest FP32 kernels between two 64-thread blocks per SM and one
+// wave: there the waiting blocks take their places unevenly (D3Q27xD3Q27 FP32
+// 24^3 2.75 against 3.05 us, but 28^3 3.57 against 3.40 and 32^3 3.80 against
+// 3.72; D3Q27xD3Q19 32^3 3.2 on some runs and up to 3.9 on others, 3.6 without).
+bool overlaps_steps(const lbm_ctx* h)
+{
+    const bool longest = h->p.storage == LBM_FP32 && h->q.qf + h->q.qg >= 46;
+    return !(longest && one_short_wave(h) && h->geo.n3 > 2u * 64u * (uint32_t)h->num_sms);
+}
+
 // Default launch shape of one AA parity, from per-parity sweeps of the
 // candidate shapes at 256^3: the two-nodes-per-thread kernel runs best in
 // 128-thread blocks of 64 x 2, except on the odd steps of D3Q27xD3Q19, where
@@ -228,12 +242,17 @@ void pick_block(const lbm_ctx* h, int odd, int& bx, int& by)
 // 72^3 25.0 / 17.0, 96^3 55.9 / 52.6, 160^3 243 / 229. Where a row fills its
 // blocks the flat order costs its division (128^3 118.2 / 119.7), hence the
 // 4 %. 128 threads against 256: up to 26 % faster, at most 2 % slower (16^3 to
-// 225 x 150 x 75, six pairs and storages).
+// 225 x 150 x 75, six pairs and storages). D3Q27xD3Q27 FP32 keeps its shape
+// up to three 64-thread blocks per SM, where idle lanes cost less than the
+// division (16^3 to 28^3 2.44, 2.51, 2.75, 3.40 us against 2.63, 2.60, 2.82,
+// 3.47; at 7 blocks per SM 33^3 5.78 against 4.43).
 int pick_flat(const lbm_ctx* h, int odd, int bx, int by)
 {
     const int row = uses_pairs(h, odd) ? h->p.nx / 2 : h->p.nx;
     const int64_t plane = (int64_t)row * h->p.ny;
     if (row < 2) return 0;
+    const int64_t blocks = (int64_t)((row + bx - 1) / bx) * ((h->p.ny + by - 1) / by) * h->p.nz;
+    if (h->p.storage == LBM_FP32 && h->q.qf + h->q.qg > 46 && blocks * bx * by <= (int64_t)(3 * 64) * h->num_sms) return 0;
     int64_t best = (int64_t)((row + bx - 1) / bx) * ((h->p.ny + by - 1) / by) * (bx * by) * 100 / 104;
     int pick = 0;
     for (int t = 128; t >= 64; t /= 2) {
@@ -558,11 +577,7 @@ cudaError_t launch_range(lbm_ctx* h, int odd, const StepRange& r, cudaStream_t s
     void* args[] = {&a};
     const int flat = h->flat[odd] ? 1 : 0;
     const void* k = uses_pairs(h, odd) ? h->ks->step2[h->p.forcing][odd][flat] : h->ks->step[h->p.forcing][odd][flat];
-    // the next step's launch overlaps this one's end (launch_dependents): 64^3
-    // FP32 D3Q27xD3Q19 11.7 against 12.2 us per step, 32^3 D3Q19xD3Q7 2.2 against
-    // 2.7. Below one wave of the longer kernels the waiting blocks share SMs with
-    // the running ones: 27x19 32^3 3.3 to 3.9 from run to run against 3.46.
-    return launch_overlapped(k, step_grid(h, odd, r), step_block(h, odd), args, s, !one_short_wave(h));
+    return launch_overlapped(k, step_grid(h, odd, r), step_block(h, odd), args, s, overlaps_steps(h));
 }
 
 cudaError_t launch_step(lbm_ctx* h, int odd, cudaStream_t s)

@@ -148,6 +148,23 @@ int halo_buffers(long short_by)
     return 0;
 }
 
+// The launches of two single steps: threads of a block, whether rows are
+// numbered through, whether the launch overlaps the one before.
+int step_launches(int nx, int ny, int nz, int pair, int storage)
+{
+    lbm_handle h = make(nx, ny, nz, pair, storage);
+    start(h);
+    g_work.clear();
+    lbm_step(h, 1);
+    lbm_step(h, 1);
+    for (const Work& w : g_work)
+        if (w.kind == Work::kLaunch)
+            std::printf("%u %s %s\n", w.launch.block.x * w.launch.block.y, w.launch.as<lbm::StepArgs>().flat ? "flat" : "shaped",
+                        w.launch.overlapped ? "overlapped" : "alone");
+    lbm_destroy(h);
+    return 0;
+}
+
 }  // namespace
 
 int main(int argc, char** argv)
@@ -160,6 +177,8 @@ int main(int argc, char** argv)
     if (what == "record") return record_scratch(std::atoi(argv[2]));
     if (what == "batch") return batch_calls(argv[2]);
     if (what == "halo") return halo_buffers(std::atol(argv[2]));
+    const auto arg = [&](int i) { return std::atoi(argv[i]); };
+    if (what == "launches") return step_launches(arg(2), arg(3), arg(4), arg(5), arg(6));
     std::printf("unknown check '%s'\n", what.c_str());
     return 2;
 }

@@ -6,7 +6,7 @@ import subprocess
 
 import pytest
 
-from paper_2605_14505_gb300 import build
+from paper_2605_14505_gb300 import build, lbm
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 
@@ -76,3 +76,25 @@ def test_halo_buffers_are_as_long_as_said(host, short_by, status, launches):
     """A buffer that ends at its last byte is taken, one that ends before it is
     refused with nothing launched."""
     assert host("halo", short_by) == [f"pack {status} unpack {status} launches {launches}"] * 4
+
+
+@pytest.mark.parametrize("n,pair,storage,even,odd", [
+    (16, "27x27", "fp32", "64 shaped overlapped", "128 shaped overlapped"),
+    (26, "27x27", "fp32", "64 shaped overlapped", "128 shaped overlapped"),   # 17576 of 19456 nodes
+    (28, "27x27", "fp32", "64 shaped alone", "128 shaped alone"),
+    (33, "27x27", "fp32", "128 flat alone", "128 flat alone"),
+    (36, "27x27", "fp32", "64 flat alone", "64 flat alone"),
+    (24, "27x19", "fp32", "64 flat overlapped", "64 flat overlapped"),
+    (32, "27x19", "fp32", "64 shaped alone", "64 shaped alone"),
+    (32, "19x19", "fp32", "64 shaped overlapped", "64 shaped overlapped"),
+    (20, "27x19", "fp16", "128 flat overlapped", "128 flat overlapped"),
+    (32, "27x27", "fp16", "128 flat overlapped", "128 flat overlapped"),
+    (31, "27x19", "bf16", "64 shaped overlapped", "64 shaped overlapped"),    # one node per thread
+    (64, "27x27", "fp32", "64 shaped overlapped", "128 shaped overlapped"),   # more than a wave
+])
+def test_launches_of_small_lattices(host, n, pair, storage, even, odd):
+    """Steps overlap their launches except FP32 pairs of 46 and more values between
+    two 64-thread blocks per SM and one wave; D3Q27xD3Q27 keeps its block shape
+    up to three such blocks per SM."""
+    storages = {"fp32": 0, "fp16": 1, "bf16": 2}
+    assert host("launches", n, n, n, lbm.PAIRS[pair], storages[storage]) == [even, odd]
