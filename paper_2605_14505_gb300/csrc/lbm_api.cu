@@ -513,7 +513,7 @@ cudaError_t launch_staged(lbm_ctx* h, int odd, int W, cudaStream_t s)
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, stage_threads(W), smem);
         if (e != cudaSuccess) return e;
         if (occ < 1) return cudaErrorInvalidConfiguration;
-        const size_t cap = (size_t)(h->num_sms > 0 ? h->num_sms : 1) * (size_t)occ;
+        const size_t cap = (size_t)h->num_sms * (size_t)occ;
         h->stage_grid = (int)(a.ntiles < cap ? a.ntiles : cap);
     }
     h->stage_used = true;
@@ -650,8 +650,8 @@ SkewPlan skew_plan(const lbm_ctx* h)
         p.jz = (int)std::min<double>(std::max(1.0, std::round(side)), std::max(1, nz / kSkewDepth));
         p.jy = (int)std::min<int64_t>((want + p.jz - 1) / p.jz, std::max(1, ny / kSkewDepth));
     }
-    // a box too flat for strips that L2 holds
-    if ((int64_t)p.jz * p.jy * 2 < want) return whole;
+    // a box too flat for strips that L2 holds, or for two of them
+    if (p.jz * p.jy == 1 || (int64_t)p.jz * p.jy * 2 < want) return whole;
     return p;
 }
 
@@ -797,7 +797,7 @@ dim3 node_grid(const lbm_ctx* h) { return dim3((h->geo.n3 + 255u) / 256u); }
 int flat_grid(const lbm_ctx* h)
 {
     size_t blocks = ((size_t)h->geo.n3 + 255) / 256;
-    size_t cap = (size_t)(h->num_sms > 0 ? h->num_sms : 132) * 16;
+    size_t cap = (size_t)h->num_sms * 16;
     return (int)(blocks < cap ? blocks : cap);
 }
 

@@ -25,11 +25,8 @@ lbm_handle make(int nx, int ny, int nz, int pair, int storage, int forcing = LBM
 
 void start(lbm_handle h)
 {
-    lbm_params p;
-    lbm_get_params(h, &p);
-    std::vector<double> ones(3 * (size_t)p.nx * p.ny * p.nz, 1.0);
-    if (lbm_init_fields(h, ones.data(), ones.data(), ones.data(), nullptr, nullptr, 0.0))
-        std::printf("init: %s\n", lbm_last_error());
+    const double field = 1.0;   // copies are recorded, not made
+    if (lbm_init_fields(h, &field, &field, &field, nullptr, nullptr, 0.0)) std::printf("init: %s\n", lbm_last_error());
 }
 
 // A record after a failed one: the k-th allocation of the first call fails, the
@@ -165,6 +162,29 @@ int step_launches(int nx, int ny, int nz, int pair, int storage)
     return 0;
 }
 
+// Step launches of a lattice for calls of the given step counts: AA parity,
+// planes and rows (first, number) and the direction; "graph" in front of a
+// replay's. `call` of a number before each call's.
+int step_ranges(int nx, int ny, int nz, int pair, int storage, int calls, char** counts)
+{
+    lbm_handle h = make(nx, ny, nz, pair, storage);
+    start(h);
+    for (int c = 0; c < calls; ++c) {
+        g_work.clear();
+        std::printf("call %s\n", counts[c]);
+        if (lbm_step(h, std::atoi(counts[c]))) std::printf("%s\n", lbm_last_error());
+        for (const Work& w : g_work) {
+            if (w.kind != Work::kLaunch) continue;
+            const lbm::StepArgs& a = w.launch.as<lbm::StepArgs>();
+            const bool odd = w.launch.is("Lb1E");
+            std::printf("%s%d %d %u %d %d %d\n", w.replayed ? "graph " : "", odd ? 1 : 0, a.z0, w.launch.grid.z, a.y0, a.rows,
+                        a.down);
+        }
+    }
+    lbm_destroy(h);
+    return 0;
+}
+
 }  // namespace
 
 int main(int argc, char** argv)
@@ -179,6 +199,7 @@ int main(int argc, char** argv)
     if (what == "halo") return halo_buffers(std::atol(argv[2]));
     const auto arg = [&](int i) { return std::atoi(argv[i]); };
     if (what == "launches") return step_launches(arg(2), arg(3), arg(4), arg(5), arg(6));
+    if (what == "steps") return step_ranges(arg(2), arg(3), arg(4), arg(5), arg(6), argc - 7, argv + 7);
     std::printf("unknown check '%s'\n", what.c_str());
     return 2;
 }

@@ -282,6 +282,7 @@ cudaError_t cudaGraphLaunch(cudaGraphExec_t x, cudaStream_t s)
 {
     for (Work w : x->work) {
         w.stream = s;
+        w.replayed = true;
         add(w);
     }
     return cudaSuccess;

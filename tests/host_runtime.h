@@ -27,6 +27,7 @@ struct Work {
     cudaStream_t stream = nullptr;
     Launch launch;
     void* at = nullptr;   // event, or destination
+    bool replayed = false;   // by a graph
 };
 
 extern std::vector<Work> g_work;

@@ -98,3 +98,24 @@ def test_launches_of_small_lattices(host, n, pair, storage, even, odd):
     up to three such blocks per SM."""
     storages = {"fp32": 0, "fp16": 1, "bf16": 2}
     assert host("launches", n, n, n, lbm.PAIRS[pair], storages[storage]) == [even, odd]
+
+
+def _calls(lines):
+    """Steps of each call and its launches (graph replay?, parity, z0, planes, y0, rows, down)."""
+    calls = []
+    for line in lines:
+        words = line.split()
+        if words[0] == "call":
+            calls.append((int(words[1]), []))
+        else:
+            calls[-1][1].append((words[0] == "graph",) + tuple(int(w) for w in words[-6:]))
+    return calls
+
+
+def test_a_box_of_one_strip_steps_whole(host):
+    """106 MB between 3/4 and 0.8 of L2 with too few planes and rows for two
+    strips: whole-lattice steps, replayed 64 to a graph from the first call."""
+    (_, launches), (_, more) = _calls(host("steps", 1000, 24, 24, 0, 0, 130, 64))
+    assert [x[0] for x in launches] == [True] * 128 + [False] * 2
+    assert [x[0] for x in more] == [True] * 64
+    assert all(x[2:6] == (0, 24, 0, 24) for x in launches + more)
