@@ -4,11 +4,15 @@ tests/host_runtime.cpp, which records the work and can fail a chosen call."""
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 from paper_2605_14505_gb300 import build, lbm
 
+from _strips import LARGE, PLANS
+
 HERE = os.path.dirname(os.path.abspath(__file__))
+STORAGES = {"fp32": 0, "fp16": 1, "bf16": 2}
 
 
 @pytest.fixture(scope="module")
@@ -96,8 +100,7 @@ def test_launches_of_small_lattices(host, n, pair, storage, even, odd):
     """Steps overlap their launches except FP32 pairs of 46 and more values between
     two 64-thread blocks per SM and one wave; D3Q27xD3Q27 keeps its block shape
     up to three such blocks per SM."""
-    storages = {"fp32": 0, "fp16": 1, "bf16": 2}
-    assert host("launches", n, n, n, lbm.PAIRS[pair], storages[storage]) == [even, odd]
+    assert host("launches", n, n, n, lbm.PAIRS[pair], STORAGES[storage]) == [even, odd]
 
 
 def _calls(lines):
@@ -119,3 +122,31 @@ def test_a_box_of_one_strip_steps_whole(host):
     assert [x[0] for x in launches] == [True] * 128 + [False] * 2
     assert [x[0] for x in more] == [True] * 64
     assert all(x[2:6] == (0, 24, 0, 24) for x in launches + more)
+
+
+@pytest.mark.parametrize("shape,pair,storage,jz,jy", PLANS + LARGE)
+def test_every_strip_follows_its_neighbours(host, shape, pair, storage, jz, jy):
+    """The library's launches of calls that end a group early, start at either
+    parity and replay the graph: no node steps before a neighbour's previous
+    step or after its next one, every node takes every step at its parity, and
+    a step takes a launch per strip."""
+    _, ny, nz = shape
+    counts = (5, 18) if shape == (512, 512, 512) else (19, 4, 37, 90, 33)
+    steps = np.zeros((nz, ny), dtype=int)
+    total, replays = 0, 0
+    for n, launches in _calls(host("steps", *shape, lbm.PAIRS[pair], STORAGES[storage], *counts)):
+        for graph, odd, z0, planes, y0, rows, _ in launches:
+            replays += graph
+            z, y = (np.arange(a, a + c) % m for a, c, m in ((z0, planes, nz), (y0, rows, ny)))
+            done = steps[np.ix_(z, y)]
+            now = done.flat[0]
+            assert (done == now).all() and now % 2 == odd
+            for dz in (-1, 0, 1):
+                for dy in (-1, 0, 1):
+                    near = steps[np.ix_((z + dz) % nz, (y + dy) % ny)]
+                    assert ((near == now) | (near == now + 1)).all()
+            steps[np.ix_(z, y)] += 1
+        total += n
+        assert (steps == total).all()
+        assert len(launches) == jz * jy * n
+    assert bool(replays) == (len(counts) > 2)
