@@ -346,9 +346,11 @@ int lbm_get_block(lbm_handle h, int* bx, int* by);
 
 /* Time each candidate launch shape on this lattice (reps even+odd step pairs
  * each, every launch timed on its own with CUDA events) and keep the fastest
- * for each AA parity. The state is saved and restored, so the simulation is
- * unchanged. best_ms_per_step (the mean of the two parities' best) may be
- * NULL. */
+ * for each AA parity. A lattice that lbm_step advances in strips is timed in
+ * strips, in groups of 16 steps (at least 2 reps of them): the shapes as set,
+ * then each candidate at both parities. The state is saved and restored, so the
+ * simulation is unchanged. best_ms_per_step (the mean of the two parities'
+ * best) may be NULL. */
 int lbm_autotune(lbm_handle h, int reps, double* best_ms_per_step);
 
 /* For FP16/BF16 storage and even nx the step kernel can update two nodes

@@ -1590,7 +1590,28 @@ int lbm_autotune(lbm_handle h, int reps, double* best_ms_per_step)
     double best[2] = {1e300, 1e300};
     int bbx[2] = {save_bx, save_bxo}, bby[2] = {save_by, save_byo}, bflat[2] = {save_flat[0], save_flat[1]};
     cudaError_t err = cudaSuccess;
+    // A lattice that lbm_step advances in strips: a launch of a strip takes a
+    // fraction of a step and starts in what the one before left in L2, so whole
+    // groups of steps are timed, with one shape at both parities and, before and
+    // after those (the first timings run on a GPU that is still speeding up), with
+    // the shapes as set.
+    const SkewPlan plan = h->l2 == L2Use::shared ? SkewPlan{1, 1, 1} : skew_plan(h);
+    const bool strips = plan.depth > 1;
+    auto time_strips = [&] {
+        const int groups = (2 * reps + plan.depth - 1) / plan.depth;   // of an even number of steps
+        for (int g = -1; g < groups && err == cudaSuccess; ++g) {      // one to warm up
+            if (g == 0) err = cudaEventRecord(ev[0], h->stream);
+            if (err == cudaSuccess) err = launch_group(h, plan, plan.depth, save_odd, (g & 1) != 0, h->stream);
+        }
+        if (err == cudaSuccess) err = cudaEventRecord(ev[1], h->stream);
+        if (err == cudaSuccess) err = cudaEventSynchronize(ev[1]);
+        float ms = 0.f;
+        if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, ev[0], ev[1]);
+        return (double)ms / (groups * plan.depth);
+    };
+    if (strips) best[0] = best[1] = time_strips();
     for (const auto& c : cand) {
+        if (err != cudaSuccess) break;
         const bool flat = c[1] == 0;
         if (flat && h->p.nx < 4) continue;               // a row of one unit has no division
         if (!flat && c[0] > 32 && c[0] / 2 >= h->p.nx) continue;  // wider than the row
@@ -1600,20 +1621,25 @@ int lbm_autotune(lbm_handle h, int reps, double* best_ms_per_step)
             h->bx = h->bxo = c[0];
             h->by = h->byo = c[1];
         }
-        // warm-up pair, then timed pairs
-        for (int s = 0; s < 2 && err == cudaSuccess; ++s) err = launch_step(h, (save_odd + s) & 1, h->stream);
-        if (err == cudaSuccess) err = cudaEventRecord(ev[0], h->stream);
-        for (int s = 0; s < 2 * reps && err == cudaSuccess; ++s) {
-            err = launch_step(h, (save_odd + s) & 1, h->stream);
-            if (err == cudaSuccess) err = cudaEventRecord(ev[s + 1], h->stream);
-        }
-        if (err == cudaSuccess) err = cudaEventSynchronize(ev[2 * reps]);
-        if (err != cudaSuccess) break;
         double t[2] = {0.0, 0.0};
-        for (int s = 0; s < 2 * reps; ++s) {
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, ev[s], ev[s + 1]);
-            t[(save_odd + s) & 1] += ms / reps;
+        if (strips) {
+            t[0] = t[1] = time_strips();
+            if (err != cudaSuccess) break;
+        } else {
+            // warm-up pair, then timed pairs
+            for (int s = 0; s < 2 && err == cudaSuccess; ++s) err = launch_step(h, (save_odd + s) & 1, h->stream);
+            if (err == cudaSuccess) err = cudaEventRecord(ev[0], h->stream);
+            for (int s = 0; s < 2 * reps && err == cudaSuccess; ++s) {
+                err = launch_step(h, (save_odd + s) & 1, h->stream);
+                if (err == cudaSuccess) err = cudaEventRecord(ev[s + 1], h->stream);
+            }
+            if (err == cudaSuccess) err = cudaEventSynchronize(ev[2 * reps]);
+            if (err != cudaSuccess) break;
+            for (int s = 0; s < 2 * reps; ++s) {
+                float ms = 0.f;
+                cudaEventElapsedTime(&ms, ev[s], ev[s + 1]);
+                t[(save_odd + s) & 1] += ms / reps;
+            }
         }
         for (int par = 0; par < 2; ++par)
             if (t[par] < best[par]) {
@@ -1623,20 +1649,32 @@ int lbm_autotune(lbm_handle h, int reps, double* best_ms_per_step)
                 bby[par] = flat ? (par ? save_byo : save_by) : c[1];
             }
     }
-    cudaMemcpyAsync(h->store, backup, bytes, cudaMemcpyDeviceToDevice, h->stream);
-    cudaError_t e2 = cudaStreamSynchronize(h->stream);
-    cudaFree(backup);
-    for (cudaEvent_t e : ev) cudaEventDestroy(e);
-    h->odd = save_odd;
-    if (err != cudaSuccess) {
+    auto as_set = [&] {
         h->flat[0] = save_flat[0];
         h->flat[1] = save_flat[1];
         h->bx = save_bx;
         h->by = save_by;
         h->bxo = save_bxo;
         h->byo = save_byo;
-        return cuda_fail(err, "autotune");
+    };
+    as_set();
+    if (strips && err == cudaSuccess) {
+        const double t = time_strips();
+        if (err == cudaSuccess && t <= best[0]) {
+            best[0] = best[1] = t;
+            for (int par = 0; par < 2; ++par) {
+                bflat[par] = save_flat[par];
+                bbx[par] = par ? save_bxo : save_bx;
+                bby[par] = par ? save_byo : save_by;
+            }
+        }
     }
+    cudaMemcpyAsync(h->store, backup, bytes, cudaMemcpyDeviceToDevice, h->stream);
+    cudaError_t e2 = cudaStreamSynchronize(h->stream);
+    cudaFree(backup);
+    for (cudaEvent_t e : ev) cudaEventDestroy(e);
+    h->odd = save_odd;
+    if (err != cudaSuccess) return cuda_fail(err, "autotune");
     if (e2 != cudaSuccess) return cuda_fail(e2, "autotune restore");
     h->flat[0] = bflat[0];
     h->flat[1] = bflat[1];
@@ -2585,8 +2623,17 @@ int lbm_batch_autotune(lbm_batch b, int reps, double* best_ms_per_step)
         // per-instance driver: every instance's own launch shape, then whole
         // 64-step graphs of all chains
         batch_sync_instances(b);
-        for (lbm_ctx* h : b->inst)
-            if ((rc = lbm_autotune(h, reps, nullptr))) break;
+        batch_build_rounds(b);
+        for (const std::vector<int>& round : b->rounds) {
+            for (int i : round) {
+                lbm_ctx* h = b->inst[i];
+                if (round.size() == 1) h->l2 = L2Use::alone;   // as batch_step_instances steps it
+                rc = lbm_autotune(h, reps, nullptr);
+                h->l2 = L2Use::shared;
+                if (rc) break;
+            }
+            if (rc) break;
+        }
         b->mode = LBM_BATCH_INSTANCES;
         batch_drop_graph(b);
         if (rc == LBM_OK) rc = lbm_batch_step(b, kBatchGraphSteps);   // warm-up, builds the graph

@@ -185,6 +185,48 @@ int step_ranges(int nx, int ny, int nz, int pair, int storage, int calls, char**
     return 0;
 }
 
+// lbm_autotune where a launch takes `nodes` x the threads' distance from
+// `threads` (and 1 more if it is not as flat as `flat`): how many of its step
+// launches cover the lattice, what it returns and what 32 steps take after it.
+int autotune(int n, int pair, int threads, int flat, int batched)
+{
+    lbm_handle h = nullptr;
+    lbm_batch b = nullptr;
+    if (batched) {
+        lbm_params p[2];
+        for (lbm_params& q : p) lbm_params_from_physics(&q, n, n, n, pair, LBM_GUO, 100.0, 1.0, 1.0, 0.04);
+        lbm_batch_create(&b, p, 2);
+        lbm_batch_init_tgv(b, 1, 0.0);
+        lbm_batch_instance(b, 1, &h);
+    } else {
+        h = make(n, n, n, pair, LBM_FP32);
+        start(h);
+    }
+    g_cost = [=](const Launch& l) {
+        if (!l.is("6k_step")) return l.is("k_batch") ? 1e6 : 0.0;
+        const lbm::StepArgs& a = l.as<lbm::StepArgs>();
+        const int off = std::abs((int)(l.block.x * l.block.y) - threads) + ((a.flat != 0) != (flat != 0) ? 1 : 0);
+        return 1e-9 * n * a.rows * l.grid.z * (1.0 + off);
+    };
+    g_work.clear();
+    double ms = 0.0;
+    if (batched ? lbm_batch_autotune(b, 3, &ms) : lbm_autotune(h, 3, &ms)) std::printf("%s\n", lbm_last_error());
+    int whole = 0, all = 0;
+    for (const Work& w : g_work)
+        if (w.kind == Work::kLaunch && w.launch.is("6k_step")) {
+            ++all;
+            whole += (int)w.launch.grid.z == n && w.launch.as<lbm::StepArgs>().rows == n;
+        }
+    g_work.clear();
+    batched ? lbm_batch_step(b, 32) : lbm_step(h, 32);
+    double spent = 0.0;
+    for (const Work& w : g_work)
+        if (w.kind == Work::kLaunch) spent += g_cost(w.launch);
+    std::printf("%d %d %.9g %.9g\n", whole, all, ms, spent / 32);
+    batched ? lbm_batch_destroy(b) : lbm_destroy(h);
+    return 0;
+}
+
 }  // namespace
 
 int main(int argc, char** argv)
@@ -200,6 +242,7 @@ int main(int argc, char** argv)
     const auto arg = [&](int i) { return std::atoi(argv[i]); };
     if (what == "launches") return step_launches(arg(2), arg(3), arg(4), arg(5), arg(6));
     if (what == "steps") return step_ranges(arg(2), arg(3), arg(4), arg(5), arg(6), argc - 7, argv + 7);
+    if (what == "autotune") return autotune(arg(2), arg(3), arg(4), arg(5), arg(6));
     std::printf("unknown check '%s'\n", what.c_str());
     return 2;
 }

@@ -150,3 +150,18 @@ def test_every_strip_follows_its_neighbours(host, shape, pair, storage, jz, jy):
         assert (steps == total).all()
         assert len(launches) == jz * jy * n
     assert bool(replays) == (len(counts) > 2)
+
+
+@pytest.mark.parametrize("n,pair,threads,flat,batched", [
+    (128, "27x19", 64, 0, 0), (129, "27x19", 128, 1, 0), (160, "19x7", 256, 0, 0), (96, "27x19", 64, 0, 1),
+    (60, "27x19", 64, 0, 0),
+])
+def test_autotune_times_what_is_stepped(host, n, pair, threads, flat, batched):
+    """Launches with a known cost: the time returned is the one of the steps after
+    it, at the cheapest shape, and a lattice that steps in strips (one alone in
+    its round of a batch too) is timed in strips only."""
+    (whole, timed, ms, spent), = (line.split() for line in host("autotune", n, lbm.PAIRS[pair], threads, flat, batched))
+    strips = n >= 96
+    assert int(timed) > 0 and (int(whole) == 0) == strips, (whole, timed)
+    assert float(ms) == pytest.approx(float(spent), rel=1e-5)
+    assert float(ms) == pytest.approx(1e-9 * n ** 3 * (2 if batched else 1), rel=1e-5)
