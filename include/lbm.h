@@ -227,6 +227,10 @@ int lbm_init_prefetched(lbm_handle h);
  * steps, bit for bit. */
 int lbm_step(lbm_handle h, int64_t nsteps);
 
+/* Kernels that this handle's step and record calls have launched so far, those
+ * replayed from graphs included (a step in strips takes one per strip). */
+int lbm_launch_count(lbm_handle h, int64_t* launches);
+
 /* Block until the handle's stream (and its prefetch copies) are idle;
  * reports asynchronous CUDA errors. */
 int lbm_synchronize(lbm_handle h);

@@ -112,7 +112,7 @@ struct lbm_ctx {
     float* diag_fields = nullptr;
     double* diag_partials = nullptr;
     int diag_rows = 0;                 // rows of kDNumSlots the partials hold
-    cudaEvent_t diag_event = nullptr;  // diagnostics copied to the host
+    cudaEvent_t diag_event = nullptr;  // totals written to diag_host
     double* diag_grad = nullptr;       // pass-2 rows, then the count of finished blocks
     double* diag_host = nullptr;       // pinned; the totals, written by the last kernel itself
     // host<->device staging
@@ -132,6 +132,8 @@ struct lbm_ctx {
     bool graphs = true;
     cudaGraphExec_t graph = nullptr;
     cudaStream_t graph_stream = nullptr;
+    int64_t launches = 0;                             // kernels of steps and records, replayed ones too
+    int64_t graph_launches = 0, skew_launches = 0;    // of a replay of `graph`, `skew_graph`
 };
 
 namespace {
@@ -287,10 +289,15 @@ void drop_graph(lbm_ctx* h)
     h->skew_graph = nullptr;
 }
 
+size_t store_need(const lbm_ctx* h)
+{
+    return (size_t)(h->q.qf + h->q.qg) * h->geo.n3 * elem_size(h->p.storage);
+}
+
 int ensure_store(lbm_ctx* h)
 {
     if (h->store) return LBM_OK;
-    size_t bytes = (size_t)(h->q.qf + h->q.qg) * h->geo.n3 * elem_size(h->p.storage);
+    const size_t bytes = store_need(h);
     void* ptr = nullptr;
     cudaError_t e = cudaMalloc(&ptr, bytes);
     if (e != cudaSuccess) {
@@ -517,6 +524,7 @@ cudaError_t launch_staged(lbm_ctx* h, int odd, int W, cudaStream_t s)
         h->stage_grid = (int)(a.ntiles < cap ? a.ntiles : cap);
     }
     h->stage_used = true;
+    ++h->launches;
     void* args[] = {&a};
     return cudaLaunchKernel(k, dim3((unsigned)h->stage_grid), dim3((unsigned)stage_threads(W)), args, smem, s);
 }
@@ -526,10 +534,6 @@ cudaError_t launch_staged(lbm_ctx* h, int odd, int W, cudaStream_t s)
 struct StepRange {
     int z0, planes, y0, rows, down;
 };
-size_t store_need(const lbm_ctx* h)
-{
-    return (size_t)(h->q.qf + h->q.qg) * h->geo.n3 * elem_size(h->p.storage);
-}
 StepRange whole_range(const lbm_ctx* h)
 {
     // a z-slab updates its own planes 1 .. nz - 2; the ghost planes are only
@@ -574,6 +578,7 @@ StepArgs step_args(lbm_ctx* h, int odd, const StepRange& r)
 cudaError_t launch_range(lbm_ctx* h, int odd, const StepRange& r, cudaStream_t s)
 {
     StepArgs a = step_args(h, odd, r);
+    ++h->launches;
     void* args[] = {&a};
     const int flat = h->flat[odd] ? 1 : 0;
     const void* k = uses_pairs(h, odd) ? h->ks->step2[h->p.forcing][odd][flat] : h->ks->step[h->p.forcing][odd][flat];
@@ -687,10 +692,12 @@ cudaError_t launch_group(lbm_ctx* h, const SkewPlan& p, int k, int odd, bool mir
 }
 
 // Captures `record` on the stream and instantiates it; null where the stream
-// cannot be captured (the caller then launches eagerly).
+// cannot be captured (the caller then launches eagerly). `launches` gets the
+// number of its kernels.
 template <class Record>
-cudaGraphExec_t capture_graph(cudaStream_t s, Record&& record)
+cudaGraphExec_t capture_graph(lbm_ctx* h, cudaStream_t s, int64_t* launches, Record&& record)
 {
+    const int64_t before = h->launches;
     cudaGraph_t g = nullptr;
     cudaGraphExec_t x = nullptr;
     cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
@@ -701,6 +708,8 @@ cudaGraphExec_t capture_graph(cudaStream_t s, Record&& record)
     }
     if (e == cudaSuccess) e = cudaGraphInstantiate(&x, g, 0);
     if (g) cudaGraphDestroy(g);
+    *launches = h->launches - before;
+    h->launches = before;
     if (e == cudaSuccess) return x;
     cudaGetLastError();
     return nullptr;
@@ -721,7 +730,7 @@ cudaError_t step_skewed(lbm_ctx* h, const SkewPlan& p, int64_t nsteps, cudaStrea
                             h->skew_eager >= kSkewGraphAfter * kSkewGraphSteps;
         if (graphs && h->odd == 0) {
             if (!h->skew_graph)
-                h->skew_graph = capture_graph(s, [&] {
+                h->skew_graph = capture_graph(h, s, &h->skew_launches, [&] {
                     const cudaError_t e = launch_group(h, p, kSkewDepth, 0, true, s);
                     return e != cudaSuccess ? e : launch_group(h, p, kSkewDepth, 0, false, s);
                 });
@@ -729,6 +738,7 @@ cudaError_t step_skewed(lbm_ctx* h, const SkewPlan& p, int64_t nsteps, cudaStrea
                 const cudaError_t e = cudaGraphLaunch(h->skew_graph, s);
                 if (e != cudaSuccess) return e;
                 h->mirrored = false;
+                h->launches += h->skew_launches;
                 h->step += kSkewGraphSteps;
                 nsteps -= kSkewGraphSteps;
                 continue;
@@ -764,9 +774,11 @@ cudaError_t launch_totals(lbm_ctx* h, DiagArgs a, int rows)
         void* args[] = {&at, &rows, &mid};
         e = launch_overlapped(diag_rows_kernel(), dim3((unsigned)h->num_sms), dim3(kDiagBlock), args, h->stream);
         if (e != cudaSuccess) return e;
+        ++h->launches;
         at = mid;
         rows = h->num_sms;
     }
+    ++h->launches;
     if (h->slab) {
         void* args[] = {&at, &rows, &a.out};
         return launch_overlapped(diag_totals_kernel(), dim3(kDiagPass1), dim3(kDiagBlock), args, h->stream);
@@ -787,6 +799,7 @@ int enqueue_diagnostics(lbm_ctx* h)
     DiagArgs a = diag_args(h);
     void* args[] = {&a};
     LBM_CUDA(cudaLaunchKernel(h->ks->diag_moments, dim3(blocks), dim3(kDiagBlock), args, 0, h->stream), "diag pass 1");
+    ++h->launches;
     LBM_CUDA(launch_totals(h, a, (int)blocks), "diag pass 2");
     return LBM_OK;
 }
@@ -1123,7 +1136,7 @@ int lbm_get_stream(lbm_handle h, void** stream)
 int lbm_required_bytes(lbm_handle h, size_t* bytes)
 {
     if (!h || !bytes) return fail(LBM_EINVAL, "null argument");
-    *bytes = (size_t)(h->q.qf + h->q.qg) * h->geo.n3 * elem_size(h->p.storage);
+    *bytes = store_need(h);
     return LBM_OK;
 }
 
@@ -1311,7 +1324,7 @@ int lbm_step(lbm_handle h, int64_t nsteps)
     while (nsteps > 0) {
         if (h->graphs && h->stream != nullptr && h->odd == 0 && nsteps >= kGraphSteps) {
             if (!h->graph)
-                h->graph = capture_graph(h->stream, [&] {
+                h->graph = capture_graph(h, h->stream, &h->graph_launches, [&] {
                     cudaError_t e = cudaSuccess;
                     for (int s = 0; s < kGraphSteps && e == cudaSuccess; ++s) e = launch_step(h, s & 1, h->stream);
                     return e;
@@ -1321,6 +1334,7 @@ int lbm_step(lbm_handle h, int64_t nsteps)
                 continue;
             }
             LBM_CUDA(cudaGraphLaunch(h->graph, h->stream), "graph launch");
+            h->launches += h->graph_launches;
             h->step += kGraphSteps;
             nsteps -= kGraphSteps;
             continue;
@@ -1383,6 +1397,7 @@ int lbm_step_diagnostics(lbm_handle h, int64_t nsteps, lbm_diag* out)
     const void* k = pairs ? h->ks->step2_diag[h->p.forcing][odd] : h->ks->step_diag[h->p.forcing][odd];
     LBM_CUDA(cudaLaunchKernel(k, grid, step_block(h, odd), args, 0, h->stream), "diagnosing step");
     const int64_t step0 = h->step;
+    ++h->launches;
     h->odd ^= 1;
     h->step += 1;
     LBM_CUDA(launch_totals(h, da, rows), "diag pass 2");
@@ -1548,6 +1563,13 @@ int lbm_step_count(lbm_handle h, int64_t* step)
     return LBM_OK;
 }
 
+int lbm_launch_count(lbm_handle h, int64_t* launches)
+{
+    if (!h || !launches) return fail(LBM_EINVAL, "null argument");
+    *launches = h->launches;
+    return LBM_OK;
+}
+
 int lbm_set_block(lbm_handle h, int bx, int by)
 {
     if (!h) return fail(LBM_EINVAL, "null handle");
@@ -1578,7 +1600,7 @@ int lbm_autotune(lbm_handle h, int reps, double* best_ms_per_step)
     static const int cand[][2] = {{32, 1}, {32, 2}, {32, 4}, {32, 8}, {64, 1}, {64, 2}, {64, 4},
                                   {128, 1}, {128, 2}, {256, 1}, {64, 0}, {128, 0}, {256, 0}};
     void* backup = nullptr;
-    size_t bytes = (size_t)(h->q.qf + h->q.qg) * h->geo.n3 * elem_size(h->p.storage);
+    const size_t bytes = store_need(h);
     LBM_CUDA(cudaMalloc(&backup, bytes), "autotune backup allocation");
     // one event between consecutive launches, so that each launch is timed
     // on its own and the two AA parities get their own best shape

@@ -129,6 +129,7 @@ _SIGS = {
     "lbm_set_populations": ([_H, _DP, _DP], ctypes.c_int),
     "lbm_sample_populations": ([_H, ctypes.POINTER(ctypes.c_int64), ctypes.c_int64, _DP, _DP],
                                ctypes.c_int),
+    "lbm_launch_count": ([_H, ctypes.POINTER(ctypes.c_int64)], ctypes.c_int),
     "lbm_step_count": ([_H, ctypes.POINTER(ctypes.c_int64)], ctypes.c_int),
     "lbm_set_block": ([_H, ctypes.c_int, ctypes.c_int], ctypes.c_int),
     "lbm_get_block": ([_H, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
@@ -417,6 +418,12 @@ def lbm_step_count(h) -> int:
     s = ctypes.c_int64()
     _check(load_library().lbm_step_count(h, ctypes.byref(s)))
     return s.value
+
+
+def lbm_launch_count(h) -> int:
+    n = ctypes.c_int64()
+    _check(load_library().lbm_launch_count(h, ctypes.byref(n)))
+    return n.value
 
 
 def lbm_set_block(h, bx: int, by: int):

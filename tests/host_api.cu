@@ -227,6 +227,27 @@ int autotune(int n, int pair, int threads, int flat, int batched)
     return 0;
 }
 
+// lbm_launch_count against the launches recorded, after each of: steps, a fused
+// record with more steps, a record.
+int launch_count(int n, int pair, int storage)
+{
+    lbm_handle h = make(n, n, n, pair, storage);
+    start(h);
+    lbm_diag d;
+    g_work.clear();
+    for (int k : {1, 70, 33, 300}) {
+        lbm_step(h, k);
+        lbm_step_diagnostics(h, k, &d);
+        lbm_diagnostics(h, &d);
+        int64_t launches = 0, recorded = 0;
+        lbm_launch_count(h, &launches);
+        for (const Work& w : g_work) recorded += w.kind == Work::kLaunch;
+        std::printf("%lld %lld\n", (long long)launches, (long long)recorded);
+    }
+    lbm_destroy(h);
+    return 0;
+}
+
 }  // namespace
 
 int main(int argc, char** argv)
@@ -243,6 +264,7 @@ int main(int argc, char** argv)
     if (what == "launches") return step_launches(arg(2), arg(3), arg(4), arg(5), arg(6));
     if (what == "steps") return step_ranges(arg(2), arg(3), arg(4), arg(5), arg(6), argc - 7, argv + 7);
     if (what == "autotune") return autotune(arg(2), arg(3), arg(4), arg(5), arg(6));
+    if (what == "count") return launch_count(arg(2), arg(3), arg(4));
     std::printf("unknown check '%s'\n", what.c_str());
     return 2;
 }

@@ -165,3 +165,11 @@ def test_autotune_times_what_is_stepped(host, n, pair, threads, flat, batched):
     assert int(timed) > 0 and (int(whole) == 0) == strips, (whole, timed)
     assert float(ms) == pytest.approx(float(spent), rel=1e-5)
     assert float(ms) == pytest.approx(1e-9 * n ** 3 * (2 if batched else 1), rel=1e-5)
+
+
+@pytest.mark.parametrize("n,pair,storage", [(32, "19x7", "fp32"), (128, "27x19", "fp32"), (64, "27x19", "fp16")])
+def test_launches_are_counted(host, n, pair, storage):
+    """Eager launches, whole and in strips, graph replays, and the passes of records
+    with and without a first sum of their rows."""
+    counts = [line.split() for line in host("count", n, lbm.PAIRS[pair], STORAGES[storage])]
+    assert all(a == b for a, b in counts) and int(counts[-1][0]) > 2 * (1 + 70 + 33 + 300)
