@@ -50,10 +50,11 @@ NCU_TRAFFIC = {"fingerprint": "18dee20ce526b74c", "fp32": 6116793728, "fp16": 30
 
 
 def source_fingerprint() -> str:
-    """Hash of the sources that define the bench's step kernels: the device
-    headers and the D3Q27xD3Q19 instantiations (the host-side launch code, the
-    staged kernel's header and the other stencil pairs' instantiations are not
-    part of it)."""
+    """Hash of the sources that define the bench's step kernels and their
+    launches: the device headers, the D3Q27xD3Q19 instantiations, the batch
+    kernels and the host code that cuts a lattice into strips (the staged
+    kernel's header and the other stencil pairs' instantiations are not part
+    of it)."""
     import hashlib
 
     h = hashlib.sha256()
@@ -61,7 +62,7 @@ def source_fingerprint() -> str:
     for name in sorted(os.listdir(csrc)):
         # the staged kernel's header does not enter the direct step kernels' code
         if (name.endswith(".cuh") and name != "lbm_stage.cuh") or name.startswith("inst_q27q19_") \
-                or name == "lbm_dispatch.h":
+                or name in ("lbm_dispatch.h", "lbm_api.cu", "lbm_batch.cu"):
             with open(os.path.join(csrc, name), "rb") as fh:
                 h.update(name.encode())
                 h.update(fh.read())

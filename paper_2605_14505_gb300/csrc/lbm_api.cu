@@ -215,8 +215,9 @@ bool overlaps_steps(const lbm_ctx* h)
 // 1.072 / 1.155 ms as 256). Below 20 waves 128 threads: the last, partly filled
 // wave then weighs less than the row order gains (27x19 / 19x7 FP32 at 64^3 11.9
 // / 7.5 us against 12.9 / 7.7 with 256, at 128^3 117.3 / 67.1 against 118.4 /
-// 67.3), and below one wave of the longer kernels 64 (27x19 Guo 32^3, 200 steps
-// and a record: 760 us; 128 757; 256 728 to 769 with where its few blocks land).
+// 67.3), and below one wave of the longer kernels 64 (27x19 Guo FP32 shaped, 64 /
+// 256 threads, us per step: 16^3 2.92 / 3.21, 24^3 3.05 / 3.40, 28^3 3.31 / 3.62,
+// 32^3 3.60 / 3.66; at 31^3, where 256 fill 124 SMs evenly, 3.89 / 3.77).
 void pick_block(const lbm_ctx* h, int odd, int& bx, int& by)
 {
     const bool pairs = uses_pairs(h, odd);
@@ -354,7 +355,8 @@ cudaError_t launch_overlapped(const void* k, dim3 grid, dim3 block, void** args,
     return cudaLaunchKernelExC(&cfg, k, args);
 }
 
-// Pass 1 on its own: four blocks per SM, or one per 256 nodes of a small lattice.
+// Pass 1 on its own: four blocks per SM (D3Q27xD3Q27, whose kernel fits three,
+// runs the fourth in a second wave), or one per 256 nodes of a small lattice.
 uint32_t moment_blocks(const lbm_ctx* h, uint32_t nodes)
 {
     return std::min(4u * (uint32_t)h->num_sms, (nodes + kDiagBlock - 1) / kDiagBlock);
@@ -591,8 +593,11 @@ cudaError_t launch_step(lbm_ctx* h, int odd, cudaStream_t s)
     if (W > 0) return launch_staged(h, odd, W, s);
     StepRange r = whole_range(h);
     // of a lattice that L2 does not hold well a step starts where the one before
-    // ended, in what is there; a smaller one keeps its blocks on their SMs (27x19
-    // Guo 32^3, 200 steps and a record: 760 us, alternating 778)
+    // ended, in what is there; a smaller one keeps its blocks on their SMs. One
+    // way / alternating, us per step of FP32 27x19 Guo: 32^3 (0.05 L2) 3.38 / 3.50,
+    // 44^3 5.80 / 5.89, 56^3 8.90 / 8.98, 64^3 (0.36) 11.94 / 11.95, 72^3 (0.51)
+    // 16.49 either way, 80^3 (0.70) 25.6 / 23.2; 19x7 32^3 2.17 / 2.31, 64^3 7.18 /
+    // 7.21
     r.down = odd && 2 * store_need(h) > h->l2_bytes;
     return launch_range(h, odd, r, s);
 }
@@ -624,12 +629,15 @@ struct SkewPlan {
 constexpr int kSkewDepth = 16;   // deeper gains under 0.3 %, and the ranges move further
 constexpr int kSkewSteps = 4;    // fewer steps in a call run whole
 
-// Strips of at most 3/4 of L2 in FP32; 0.4 of it for lattices of up to 6 L2,
-// which are stepped beside others (several handles on their streams) more often
-// and then still share it: 50 steps and a record at 128^3 in strips of 0.4 /
-// 0.75 of L2 5.13 / 4.98 ms alone and 5.29 / 5.61 beside another lattice
-// (whole-lattice steps 5.44 and 5.60), 100 at 256^3 88.5 / 82.9 alone and 84.9 /
-// 88.5 beside (89.5 and 90.1), at 160^3 as good either way. One L2 in 16 bits,
+// Strips of at most 3/4 or 0.4 of L2 in FP32. Alone on the GPU the larger ones
+// are the faster, beside another lattice stepped on its own stream, which then
+// shares L2, the smaller: 50 steps and a record at 128^3 in strips of 0.4 / 0.75
+// of L2 5.13 / 4.98 ms alone and 5.29 / 5.61 beside another (whole-lattice steps
+// 5.44 and 5.60), 100 at 256^3 88.5 / 82.9 alone and 84.9 / 88.5 beside (89.5 and
+// 90.1), at 160^3 as good either way. Which it is, a handle does not know (but for
+// an instance with a round of its batch to itself): lattices of up to 6 L2 take
+// the smaller strips, of which several are likelier to be stepped at a time, and
+// no faster choice was measured between 160^3 and 256^3. One L2 in 16 bits,
 // where only deep strips gain (256^3 in 96 / 129 MB strips 449.7 / 446.4 us per
 // step). Along z alone while the strips are 16 planes thick, else about square
 // in y and z.

@@ -4,9 +4,10 @@
 // so as one copy per run an exchange of two slabs is 112 copies a phase, bound
 // by their launches (64 KB each at 128^2). 20 steps of a 128^3 FP32 lattice in
 // two slabs: 9.34 ms with a copy per run and host waits between the slabs,
-// 2.72 ms with these launches ordered by the slabs' streams. Here grid.y is the run and grid.z the side; a run
-// is a plain coalesced copy of the widest type that the alignment allows, four
-// independent loads a thread before their stores.
+// 2.48 ms with these launches ordered by the slabs' streams (and the steps'
+// own gains). Here grid.y is the run and grid.z the side; a run is a plain
+// coalesced copy of the widest type that the alignment allows, four independent
+// loads a thread before their stores.
 #include <cuda_runtime.h>
 
 #include "lbm_halo.cuh"

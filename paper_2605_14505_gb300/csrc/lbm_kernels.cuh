@@ -379,8 +379,8 @@ __device__ __forceinline__ int step_plane(const StepArgs& a)
 // stores, the next step's blocks may take free SM slots; they wait there until
 // this launch is complete and its stores visible, so only the launch itself
 // overlaps. Asked for at the start of a step instead, the waiting blocks crowd
-// the few free SMs of a small lattice (D3Q27xD3Q19 32^3 5.4 against 3.3 us per
-// step; 3.5 without overlap). Without the launch attribute both are no-ops.
+// the few free SMs of a small lattice (D3Q27xD3Q19 32^3 5.4 against 3.2 us per
+// step; 3.6 without overlap). Without the launch attribute both are no-ops.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -1145,8 +1145,9 @@ __global__ void k_set_pops(PopArgs a)
     }
 }
 
-// Pass 1 on its own: four 256-thread blocks per SM, all of them resident, that
-// stride over the lattice; thread t sums nodes t, t + stride, ... in order.
+// Pass 1 on its own: four 256-thread blocks per SM that stride over the lattice,
+// all of them resident (three for D3Q27xD3Q27, whose 54 values a node do not fit
+// 64 registers); thread t sums nodes t, t + stride, ... in order.
 // The sums live in shared memory: in registers they kept three blocks on an SM
 // (80 registers), so the fourth ran alone in a second wave. A block's warps
 // stay together: with the loads' 256-byte prefetch a warp also fetches its
