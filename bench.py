@@ -42,20 +42,21 @@ METRIC = "DDF MLUPS (FP32 storage) & % of HBM roofline; FP16-storage vs FP32 at 
 WORKLOAD = "stratified TGV 256^3, D3Q27xD3Q19, velocity-shift (Shan-Chen) forcing, Re 800, Fr 0.1, Pr 1, U0 0.04"
 
 
-# DRAM bytes per step-kernel launch on the 256^3 bench lattice
-# (dram__bytes_read.sum + dram__bytes_write.sum from one ncu capture, mean of
-# an even and an odd launch), with the fingerprint of the kernel sources the
-# capture ran; reported as null once the sources differ from it.
-NCU_TRAFFIC = {"fingerprint": "18dee20ce526b74c", "fp32": 6116793728, "fp16": 3027879552, "bf16": 3028134272}
+# DRAM bytes per lattice step of the 256^3 bench lattice as lbm_step runs it, in
+# skewed strips (dram__bytes_read.sum + dram__bytes_write.sum over one 16-step
+# group of strips, L2 kept from launch to launch), with the fingerprint of the
+# sources the capture ran; reported as null once the sources differ from it.
+NCU_TRAFFIC = {"fingerprint": "dc67b9c2fddd7f73", "fp32": 2226478512, "fp16": 1654111920, "bf16": 1652928928}
 
 
 def source_fingerprint() -> str:
     """Hash of the sources that define the bench's step kernels and their
     launches: the device headers, the D3Q27xD3Q19 instantiations, the batch
-    kernels and the host code that cuts a lattice into strips (the staged
-    kernel's header and the other stencil pairs' instantiations are not part
-    of it)."""
+    kernels and the host code that cuts a lattice into strips, without their
+    line comments (the staged kernel's header and the other stencil pairs'
+    instantiations are not part of it)."""
     import hashlib
+    import re
 
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2605_14505_gb300", "csrc")
@@ -63,25 +64,36 @@ def source_fingerprint() -> str:
         # the staged kernel's header does not enter the direct step kernels' code
         if (name.endswith(".cuh") and name != "lbm_stage.cuh") or name.startswith("inst_q27q19_") \
                 or name in ("lbm_dispatch.h", "lbm_api.cu", "lbm_batch.cu"):
-            with open(os.path.join(csrc, name), "rb") as fh:
+            with open(os.path.join(csrc, name), encoding="utf-8") as fh:
                 h.update(name.encode())
-                h.update(fh.read())
+                h.update(re.sub(r"[ \t]*//[^\n]*", "", fh.read()).encode())
     return h.hexdigest()[:16]
 
 
-# DRAM bytes per step of the 64-instance sweep, by driver (ncu, on the step
-# kernels of the fingerprint above): the per-instance driver over 128
-# graph-replayed steps as one profiler range (--replay-mode app-range, all
-# streams together: 739.9 GB in 128 steps, the instances' own L2 reuse
-# included); the persistent driver from one launch of 4 steps (5.97 GB per
-# step, the algorithmic 5.95 GB).
-NCU_BATCH_DRAM = {"fingerprint": "18dee20ce526b74c", "instances": 5780572946, "persistent": 5971162432}
+# DRAM bytes per step of the 64-instance sweep, by driver (ncu, sources of the
+# fingerprint): the per-instance driver over 128 steps as one profiler range
+# (--replay-mode app-range, all streams together: 268.3 GB); the persistent
+# driver from one launch of 4 steps (5.98 GB per step, the algorithmic 5.95 GB).
+NCU_BATCH_DRAM = {"fingerprint": "dc67b9c2fddd7f73", "instances": 2095939688, "persistent": 5976947904}
 
 
 def ncu_traffic(storage: str):
     if NCU_TRAFFIC["fingerprint"] != source_fingerprint():
         return None
     return NCU_TRAFFIC.get(storage)
+
+
+def strip_roofline(storage: str, n3: int, step_ms: float, peak: float) -> dict:
+    """One 256^3 step against the HBM copy rate: achieved and frac count the DRAM
+    bytes of a step (ncu), the _algorithmic figures every population read and
+    written once, most of which strips serve from L2."""
+    dram, algorithmic = ncu_traffic(storage), bytes_per_node(storage) * n3
+    rate = algorithmic / (step_ms * 1e-3) / 1e9
+    return {"bound": "issue (strips step from L2)",
+            "achieved": None if dram is None else round(dram / (step_ms * 1e-3) / 1e9, 1), "peak": peak, "unit": "GB/s",
+            "frac": None if dram is None else round(dram / (step_ms * 1e-3) / 1e9 / peak, 4), "traffic": dram,
+            "achieved_algorithmic": round(rate, 1), "frac_algorithmic": round(rate / peak, 4),
+            "algorithmic_bytes_per_step": algorithmic}
 
 
 def bytes_per_node(storage: str) -> int:
@@ -261,7 +273,6 @@ def run_gpu_arm(args):
     clk = clocks.stop()
     secs = max_over_ranks(world, secs)
     value = aggregate_mlups(float(n3) * DIAG_EVERY * args.steps, world, secs)
-    achieved = bytes_per_node("fp32") * n3 / (step_ms * 1e-3) / 1e9
     sim.close()
 
     variants = {}
@@ -270,14 +281,11 @@ def run_gpu_arm(args):
         vsecs, vstep_ms, _, dv, _ = timed(s, args.steps, args.warmup)
         vsecs = max_over_ranks(world, vsecs)
         vmlups = aggregate_mlups(float(n3) * DIAG_EVERY * args.steps, world, vsecs)
-        vach = bytes_per_node(storage) * n3 / (vstep_ms * 1e-3) / 1e9
         err = {k: abs(dv[k] - d32[k]) / abs(d32[k]) for k in ("Ek", "Ep", "eps_k", "eps_p")}
         variants[storage] = {
             "mlups": round(vmlups, 1), "speedup_vs_fp32": round(vmlups / value, 3),
             "step_kernel_ms": round(vstep_ms, 4),
-            "roofline": {"bound": "hbm", "achieved": round(vach, 1), "peak": peak, "unit": "GB/s",
-                         "frac": round(vach / peak, 4), "traffic": ncu_traffic(storage),
-                         "algorithmic_bytes_per_launch": bytes_per_node(storage) * n3},
+            "roofline": strip_roofline(storage, n3, vstep_ms, peak),
             "rel_dev_vs_fp32_gpu_at_last_timed_step": {k: float(f"{v:.3e}") for k, v in err.items()},
             "bytes_per_node": bytes_per_node(storage),
         }
@@ -339,12 +347,11 @@ def run_gpu_arm(args):
                    "storage": "fp32", "updates_per_step": DIAG_EVERY, "diagnostics_per_step": 1,
                    "parallelism": "replicas" if world > 1 else "single",
                    "l2": "inputs larger than L2 (3.09 GB store vs 129 MB L2)", "block": [bx, by]},
-        "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
-                     "frac": round(achieved / peak, 4), "traffic": ncu_traffic("fp32"),
-                     "algorithmic_bytes_per_launch": bytes_per_node("fp32") * n3,
-                     "kernel": "k_step<27x19, SC, f32> (even/odd AA)", "peak_kind": peak_kind,
-                     "counts": "achieved: algorithmic bytes (every population read and written once per step); "
-                               "steps run in strips that stay in L2, so it can exceed the HBM copy rate",
+        "roofline": {**strip_roofline("fp32", n3, step_ms, peak),
+                     "kernel": "k_step<27x19, SC, f32> (even/odd AA), a launch per strip", "peak_kind": peak_kind,
+                     "counts": "achieved / frac: DRAM bytes per step (ncu, traffic) over the measured step time; "
+                               "*_algorithmic: every population read and written once per step, which can exceed "
+                               "the HBM copy rate",
                      "bytes_per_node": bytes_per_node("fp32"), "step_kernel_ms": round(step_ms, 4),
                      "diagnosing_step_ms": round(diag_ms, 4)},
         "storage_variants": variants,
@@ -482,7 +489,8 @@ def run_batch_sweep(args, peak, world=1, rank=0):
     drivers = {0: "persistent", 1: "per_step", 2: "instances"}
     driver = drivers[cfg["mode"]]
     dram = NCU_BATCH_DRAM.get(driver) if NCU_BATCH_DRAM["fingerprint"] == source_fingerprint() else None
-    roof = {"bound": "hbm", "achieved": None, "peak": peak, "unit": "GB/s", "frac": None,
+    # in rounds that L2 holds the per-instance driver is bound by issue, the others by HBM
+    roof = {"bound": "issue" if driver == "instances" else "hbm", "achieved": None, "peak": peak, "unit": "GB/s", "frac": None,
             "traffic": dram, "algorithmic_bytes_per_step": nbytes,
             "achieved_algorithmic": round(achieved, 1), "frac_algorithmic": round(achieved / peak / world, 4),
             "counts": "achieved / frac: DRAM bytes per step (ncu, traffic) over the measured step time; "
@@ -619,7 +627,8 @@ def run_ncu_case(args):
     lbm.lbm_set_pairing(sim.h, args.ncu_pairing)
     lbm.lbm_set_tile_staging(sim.h, args.ncu_staging)
     sim.init_tgv(seed=1, noise_amp=1e-3)
-    sim.step(args.ncu_steps)
+    for _ in range(args.ncu_steps):
+        sim.step(1)   # whole-lattice launches (longer calls on large lattices run in strips)
     d = sim.diagnostics()
     sim.close()
     torch.cuda.synchronize()

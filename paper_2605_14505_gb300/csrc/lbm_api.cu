@@ -195,8 +195,8 @@ bool one_short_wave(const lbm_ctx* h) { return h->q.qf + h->q.qg >= 38 && step_w
 // Not for the longest FP32 kernels between two 64-thread blocks per SM and one
 // wave: there the waiting blocks take their places unevenly (D3Q27xD3Q27 FP32
 // 24^3 2.75 against 3.05 us, but 28^3 3.57 against 3.40 and 32^3 3.80 against
-// 3.72; D3Q27xD3Q19 32^3 3.2 to 3.3 against 3.4 to 3.6 on some boxes, up to 3.9
-// on another).
+// 3.72; D3Q27xD3Q19 32^3 3.2 to 3.3 against 3.4 to 3.6 on some GPUs, up to 3.9 on
+// another).
 bool overlaps_steps(const lbm_ctx* h)
 {
     const bool longest = h->p.storage == LBM_FP32 && h->q.qf + h->q.qg >= 46;
