@@ -49,6 +49,26 @@ def test_strips_equal_whole_steps(shape, pair, storage):
     strips.close()
 
 
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+def test_strips_of_the_256_cubed_lattice(storage):
+    """6 x 6 and 12 x 1 strips, a call that fills two groups and one that ends one early."""
+    import torch
+
+    p = lbm.lbm_params_from_physics(256, 256, 256, "27x19", "sc", 800.0, 0.1, 1.0, 0.04)
+    whole, strips = (lbm.Simulation(p, storage=storage) for _ in range(2))
+    for sim in (whole, strips):
+        sim.init_tgv(1, 1e-3)
+    for _ in range(37):
+        whole.step(1)
+    strips.step(32)
+    strips.step(5)
+    whole.synchronize()
+    strips.synchronize()
+    assert torch.equal(whole._store, strips._store)
+    whole.close()
+    strips.close()
+
+
 def test_strips_of_planes_and_rows_from_a_graph():
     """128 eager steps, then replays from both parities."""
     import torch
