@@ -490,8 +490,8 @@ def run_batch_sweep(args, peak, world=1, rank=0):
     driver = drivers[cfg["mode"]]
     dram = NCU_BATCH_DRAM.get(driver) if NCU_BATCH_DRAM["fingerprint"] == source_fingerprint() else None
     # in rounds that L2 holds the per-instance driver is bound by issue, the others by HBM
-    roof = {"bound": "issue" if driver == "instances" else "hbm", "achieved": None, "peak": peak, "unit": "GB/s", "frac": None,
-            "traffic": dram, "algorithmic_bytes_per_step": nbytes,
+    roof = {"bound": "issue" if driver == "instances" else "hbm", "achieved": None, "peak": peak, "unit": "GB/s",
+            "frac": None, "traffic": dram, "algorithmic_bytes_per_step": nbytes,
             "achieved_algorithmic": round(achieved, 1), "frac_algorithmic": round(achieved / peak / world, 4),
             "counts": "achieved / frac: DRAM bytes per step (ncu, traffic) over the measured step time; "
                       "*_algorithmic: every population read and written once per step"}
